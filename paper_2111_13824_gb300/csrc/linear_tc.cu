@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(LTHREADS, 1)
 
     if (warp == LEPI_WARPS) {
         // ---- TMA producer: stage it % LST holds step it; it is issued once step it - LST was consumed
-        if (lane == 0) {
+        if (elect_one()) {
             uint32_t it = 0;
             bool ok = true;
             for (int64_t t = t_begin; t < t_end && ok; ++t) {
@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(LTHREADS, 1)
         __syncwarp();
     } else if (warp == LEPI_WARPS + 1) {
         // ---- MMA issuer: chunk gc accumulates in tensor-memory buffer gc % 2
-        if (lane == 0) {
+        if (elect_one()) {
             uint32_t it = 0, gc = 0, commits = 0;
             bool ok = true;
             for (int64_t t = t_begin; t < t_end && ok; ++t) {

@@ -806,7 +806,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
         auto last_head = [](const TileInfo &t) { return t.nsplit < t.rows ? t.h0 + 1 : t.h0; };
         TileInfo ti = tile_info<PACK>(t_begin, L, p.BH, tpb);
         TileInfo tp = ti;  // the previous tile
-        if (warp == TCOPY_WARP && lane == 0 && ncta_tiles > 0) {
+        if (warp == TCOPY_WARP && elect_one() && ncta_tiles > 0) {
             prefetch_l2(p.v + (size_t)ti.h0 * L * TD, (uint32_t)(L * TD));
             if (last_head(ti) != ti.h0) prefetch_l2(p.v + (size_t)last_head(ti) * L * TD, (uint32_t)(L * TD));
             const uint32_t bl = (uint32_t)(ti.rows * p.ld);
@@ -833,7 +833,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
                 tp = ti;
                 ti = next_tile<PACK>(ti, L, total);
             }
-            if (warp == TCOPY_WARP && lane == 0 && it + 1 < ncta_tiles) {
+            if (warp == TCOPY_WARP && elect_one() && it + 1 < ncta_tiles) {
                 // the next tile's logits as soon as every softmax thread holds this tile's
                 const TileInfo tn = next_tile<PACK>(ti, L, total);
                 if (mbar_wait(&sh.lfree, it & 1, abort_flag)) {
@@ -869,7 +869,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
             if (!ok) *ew_stop = 1;
             epi_bar();  // D read, B written: this tile's MMAs may run
             if (*ew_stop) break;
-            if (warp == TMMA_WARP && lane == 0) {
+            if (warp == TMMA_WARP && elect_one()) {
                 if (mbar_wait(&sh.afull, it & 1, abort_flag)) {
                     tc_fence_after();
                     const uint64_t ones = smem_desc_plain(sa(ONES), 128, 256);
@@ -903,9 +903,9 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
                 read_out(ti);
             }
         }
-        if (warp == TCOPY_WARP && lane == 0 && ncopies > 0)  // no copy may land after the CTA exits
+        if (warp == TCOPY_WARP && elect_one() && ncopies > 0)  // no copy may land after the CTA exits
             mbar_wait(&sh.lload, (ncopies - 1) & 1, abort_flag, false);
-        if (warp == TMMA_WARP && lane == 0) {  // every MMA issued has completed before tensor memory is freed
+        if (warp == TMMA_WARP && elect_one()) {  // every MMA issued has completed before tensor memory is freed
             mma_commit(&sh.fin);
             mbar_wait(&sh.fin, 0, abort_flag, false);
         }

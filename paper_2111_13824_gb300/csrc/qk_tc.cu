@@ -24,10 +24,9 @@
 //     write the bytes into a staging buffer (or, for strides the tensor store
 //     cannot take, into a shared-memory tile of the output that all of them
 //     copy out with coalesced 16-byte stores);
-//   warp 16, lane 0: the bulk copies of the next tile's Q and head's K and the
-//     MMAs (a tcgen05.mma holds its issuing thread about 200 cycles, so it does
-//     nothing else);
-//   warp 17, lane 0: the tensor stores of the staging buffers.
+//   warp 16, one elected lane: the bulk copies of the next tile's Q and head's K
+//     and the MMAs (64 cycles each at N = 128, so it does nothing else);
+//   warp 17, one elected lane: the tensor stores of the staging buffers.
 // They meet only on mbarriers (chunk computed / read, staging written / read,
 // operands converted), so no warp waits at a block barrier for another's MMA
 // issue.  Every wait is bounded: after two seconds the kernel records a timeout
@@ -352,7 +351,7 @@ __global__ void __launch_bounds__(QBOUND, 1)
         }
     } else if (warp == QMMA_WARP) {
         // ---------------- warp 16, lane 0: the operand copies (BULK) and the MMAs
-        if (lane == 0) {
+        if (elect_one()) {
             // instruction descriptor: D f32, A/B f16 K-major, M = 128, N = n
             auto idesc = [](int n) -> uint32_t {
                 return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(QM >> 4) << 24);
@@ -415,7 +414,7 @@ __global__ void __launch_bounds__(QBOUND, 1)
                 mbar_wait(&sh.fin, 0, abort_flag, false);
             }
         }
-    } else if (BULK && lane == 0) {
+    } else if (BULK && elect_one()) {
         // ---------------- warp 17, lane 0: the tensor stores of the chunks' staging buffers
         uint32_t gc = 0;
         bool ok = true;

@@ -115,6 +115,17 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
     return d;
 }
 
+// One lane of a converged warp.  The code generator knows that a branch on it has a single thread, so the
+// tcgen05 and TMA instructions inside take their uniform operands directly; under "lane == 0" it serializes
+// over the lanes that might be active (measured alone, a tcgen05.mma with A in tensor memory and N = 64: 46
+// cycles to issue under lane == 0, 32 under elect, which is the instruction's own time; N = 32: 46 and 16).
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{ .reg .pred p; .reg .b32 r; elect.sync r|p, 0xffffffff; selp.u32 %0, 1, 0, p; }" : "=r"(p));
+    return p != 0;
+}
+
 __device__ __forceinline__ void mma_commit(uint64_t *b)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(sa(b))
