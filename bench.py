@@ -77,8 +77,7 @@ def tensor_peak():
 
 def bench_linear(fqvit, cfg, dev):
     """The block's four MinMax Linear layers (QKV, projection, fc1, fc2) of layer 0 at the
-    config's token count, each call (the fp16 copy of X, then the tensor-core product and its
-    requantization) timed alone with CUDA events: 10 calls after 3."""
+    config's token count, each call (the tensor-core product and its requantization) timed alone with CUDA events: 10 calls after 3."""
     peak, kind = tensor_peak()
     out, tot_ms, tot_flop = {}, 0.0, 0
     for k in synth.LINEAR_KINDS:
@@ -108,7 +107,7 @@ def bench_linear(fqvit, cfg, dev):
     out["block"] = {"ms": round(tot_ms, 5), "tflops": round(tf, 1), "frac": round(tf / peak, 4),
                     "peak_tflops": peak, "peak_source": f"{kind} (MEASURED_PEAKS.json bf16_tflops)"
                     if kind == "measured" else "fallback"}
-    out["how"] = ("fqvit_linear_q per layer of block 0 (fp16 copy of X + tcgen05 product + per-channel "
+    out["how"] = ("fqvit_linear_q per layer of block 0 (tcgen05 product + per-channel "
                   "requantization), 10 calls after 3, outside the timed step; FLOP = 2 M N K")
     return out
 

@@ -396,9 +396,8 @@ FQVIT_API int fqvit_qk_lis_attention(const int8_t *q, int64_t ld_q, int32_t zp_q
 FQVIT_API int fqvit_linear_pack_weight(const int8_t *w, int32_t N, int32_t K, int64_t ld_w, uint16_t *w_h,
                                        void *stream);
 
-/* Bytes of workspace fqvit_linear_q needs: the fp16 copy of the activations
- * (M x K x 2, rounded up to 256) and 4096 int32 per-channel weight sums.
- * 0 for a bad shape. */
+/* Bytes of workspace fqvit_linear_q asks for: M x K x 2, rounded up to 256, and
+ * 16 KB.  0 for a bad shape. */
 FQVIT_API size_t fqvit_linear_workspace_size(int64_t M, int32_t K);
 
 /*
@@ -415,12 +414,10 @@ FQVIT_API size_t fqvit_linear_workspace_size(int64_t M, int32_t K);
  * x [M][ld_x] uint8 (device); w_h [N][K] from fqvit_linear_pack_weight;
  * s_w [N] float and bias_opt [N] int32 (device; bias NULL = none);
  * y [M][ld_y] uint8 (device, caller-owned); acc_opt [M][ld_acc] int32
- * (device, may be NULL) receives acc; workspace (device, caller-owned, at
- * least fqvit_linear_workspace_size(M, K) bytes, 16-byte aligned) is
- * overwritten.  Three launches on `stream`: the per-channel weight sums, the
- * fp16 copy of x - 128 (the product runs on x - 128 and adds
- * (128 - zp_x) sum_k w[n][k] to the bias, the same integer), then the
- * tensor-core product and its requantization.
+ * (device, may be NULL) receives acc; workspace: device, caller-owned, at
+ * least fqvit_linear_workspace_size(M, K) bytes, 16-byte aligned.  One launch
+ * on `stream`; the workspace is written only when y or acc_opt overlaps x (it
+ * then receives a copy of x first).
  * Supported: K <= 16384 a multiple of 8, N <= 4096 a multiple of 16,
  * ld_x a multiple of 8 with an 8-byte aligned base, ld_y a multiple of 16 and
  * ld_acc of 4 with 16-byte aligned bases, zero points in 0..255.  Errors:

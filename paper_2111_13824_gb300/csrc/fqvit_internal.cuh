@@ -208,11 +208,11 @@ struct LinearArgs {
     int64_t ld_y;
     int32_t *acc;  // may be NULL
     int64_t ld_acc;
-    uint16_t *xh;  // workspace: fp16 [M][K]
+    uint16_t *xh;  // workspace: a copy of x when an output overlaps it
 };
 bool linear_supported(const LinearArgs &a);
 cudaError_t launch_linear(const LinearArgs &a, cudaStream_t st);
-// Workspace of launch_linear: the fp16 copy of x (M K 2 bytes, rounded up to 256) and 4096 int32 weight sums.
+// Workspace of launch_linear: M K 2 bytes, rounded up to 256, and 16 KB (used only when an output overlaps x).
 size_t linear_workspace_bytes(int64_t M, int K);
 cudaError_t launch_linear_pack_weight(const int8_t *w, int N, int K, int64_t ld_w, uint16_t *w_h, cudaStream_t st);
 cudaError_t read_clear_linear_status(int *status);
