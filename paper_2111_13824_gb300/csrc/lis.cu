@@ -1,5 +1,8 @@
 // lis.cu -- Log-Int-Softmax (supplement Algorithms 1-2, Eqs. 16-17, 33) and
-// the BitShift attention times values (Eq. 15) on CUDA cores.
+// the BitShift attention times values (Eq. 15) on CUDA cores: the softmax and
+// the product on their own (codes in memory), the fused form where no
+// tensor-core kernel takes the shape (codes written too, a mask without a bias,
+// windows above 256 keys, unaligned rows), and the choice between them.
 //
 // i-exp.  For a logit scale s the values e(q~) for every q~ in [-287, 0]
 // (int8 logits, plus an int8 relative-position bias) are tabulated in
@@ -337,11 +340,15 @@ int attention_path_override()
     return 0;
 }
 
+// The short-row kernel, the long-row kernel that keeps a whole tile's operands, the general one (us at
+// 785 keys, 96 heads, d = 64: general 78, CUDA cores 1129; at 144 keys with bias and mask, 1536 heads: 69
+// and 440), CUDA cores.  Where two take a shape the first is the faster: it does less per key.
 cudaError_t launch_lis_attention(const LisArgs &la, const AttnVArgs &a, cudaStream_t st)
 {
     const int path = attention_path_override();
     if (path == 0 && lis_attention_win_eligible(la, a)) return launch_lis_attention_win(la, a, st);
     if (path != 1 && lis_attention_tc_eligible(la, a)) return launch_lis_attention_tc(la, a, st);
+    if (path != 1 && lis_attention_gen_eligible(la, a)) return launch_lis_attention_gen(la, a, st);
     return la.bias ? fused_dispatch<true>(la, a, st) : fused_dispatch<false>(la, a, st);
 }
 

@@ -999,6 +999,10 @@ cudaError_t read_clear_device_status(int *status, cudaStream_t st)
     e = read_clear_win_status(&wst);
     if (e != cudaSuccess) return e;
     if (*status == 0) *status = wst;
+    int gst = 0;
+    e = read_clear_gen_status(&gst);
+    if (e != cudaSuccess) return e;
+    if (*status == 0) *status = gst;
     int qst = 0;
     e = read_clear_qk_status(&qst);
     if (e != cudaSuccess) return e;
