@@ -57,15 +57,29 @@ int sm_count()
     return cached[dev];
 }
 
-cudaError_t check_smem_fits(const void *kernel, size_t dynamic)
+cudaError_t prepare_smem(const void *kernel, size_t dynamic, SmemReady &ready)
 {
-    cudaFuncAttributes fa;
-    cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    int dev = 0, optin = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    const bool known = dev >= 0 && dev < 64;
+    if (known && ready[dev].load(std::memory_order_relaxed) > dynamic) return cudaSuccess;
+    cudaFuncAttributes fa;
+    if ((e = cudaFuncGetAttributes(&fa, kernel)) != cudaSuccess) return e;
+    int optin = 0;
     if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
-    return fa.sharedSizeBytes + dynamic <= (size_t)optin ? cudaSuccess : cudaErrorInvalidConfiguration;
+    if (fa.sharedSizeBytes + dynamic > (size_t)optin) return cudaErrorInvalidConfiguration;
+    // threads may race here: each sets the limit to the whole opt-in room, so none lowers another's
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
+    if (e == cudaSuccess && known)
+        ready[dev].store((uint32_t)(optin - (int)fa.sharedSizeBytes) + 1, std::memory_order_relaxed);
+    return e;
+}
+
+void forget_smem(SmemReady &ready)
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64) ready[dev].store(0, std::memory_order_relaxed);
 }
 
 int record_error(int code, const char *msg)

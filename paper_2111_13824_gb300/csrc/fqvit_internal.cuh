@@ -5,15 +5,38 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 namespace fqvit {
 
 // Number of SMs of the current device (cached per device).
 int sm_count();
 
-// Launch check of a kernel's shared memory: the compiled static size (as the runtime reports it,
-// not an estimate) plus `dynamic` bytes within the device's opt-in limit per block.  Returns
-// cudaErrorInvalidConfiguration when they do not fit, or the runtime's error.
-cudaError_t check_smem_fits(const void *kernel, size_t dynamic);
+// Bytes of dynamic shared memory (plus one) a kernel has been checked and configured for, per device;
+// one static object per kernel, zero at start.
+using SmemReady = std::atomic<uint32_t>[64];
+
+// Checks that a kernel's compiled static shared memory (as the runtime reports it, not an estimate) plus
+// `dynamic` bytes fit the device's opt-in limit per block and raises its dynamic limit to that.  Both are
+// done once per kernel, device and larger size (0.9 us of an LN call's 3.9 us on the host when done on
+// every call).  Returns cudaErrorInvalidConfiguration when they do not fit, or the runtime's error.
+cudaError_t prepare_smem(const void *kernel, size_t dynamic, SmemReady &ready);
+void forget_smem(SmemReady &ready);
+
+// Prepares and launches; a launch refused with an invalid value (the device's context was reset since
+// the kernel was configured) is prepared anew and tried once more.
+template <typename Launch>
+cudaError_t launch_prepared(const void *kernel, size_t dynamic, SmemReady &ready, Launch &&launch)
+{
+    for (int attempt = 0;; ++attempt) {
+        cudaError_t e = prepare_smem(kernel, dynamic, ready);
+        if (e != cudaSuccess) return e;
+        e = launch();
+        if (e != cudaErrorInvalidValue || attempt > 0) return e;
+        (void)cudaGetLastError();
+        forget_smem(ready);
+    }
+}
 
 // Programmatic dependent launch.  The step's kernels are launched with programmatic stream
 // serialization: the next kernel's CTAs may start (and run their set-up: barriers, tensor

@@ -699,11 +699,10 @@ cudaError_t stage_launch(const LnArgs &a, cudaStream_t st)
 {
     StageShape sh;
     if (!stage_shape(a, S, R, sh)) return cudaErrorNotSupported;
-    cudaError_t e = check_smem_fits((const void *)ln_stage_kernel<S, R>, sh.smem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(ln_stage_kernel<S, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh.smem);
-    if (e != cudaSuccess) return e;
-    return launch_pdl(ln_stage_kernel<S, R>, dim3(sh.grid), dim3(32 * sh.warps), sh.smem, st, a, sh.seg_stride);
+    static SmemReady ready;
+    return launch_prepared((const void *)ln_stage_kernel<S, R>, sh.smem, ready, [&] {
+        return launch_pdl(ln_stage_kernel<S, R>, dim3(sh.grid), dim3(32 * sh.warps), sh.smem, st, a, sh.seg_stride);
+    });
 }
 
 // Rows per segment: the most (4, 2, 1) whose warp groups still give at least half of the grid's

@@ -765,10 +765,7 @@ cudaError_t linear_launch_as(const LinParams &p, const CUtensorMap &tw, const CU
                              const CUtensorMap &ty, int grid, cudaStream_t st)
 {
     const size_t smem = T::SMEM;
-    cudaError_t e = check_smem_fits((const void *)linear_tc_kernel<T, ACC>, smem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(linear_tc_kernel<T, ACC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    static SmemReady ready;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3(LTHREADS);
@@ -783,7 +780,8 @@ cudaError_t linear_launch_as(const LinParams &p, const CUtensorMap &tw, const CU
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = T::CG > 1 ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, linear_tc_kernel<T, ACC>, p, tw, tx, ty);
+    return launch_prepared((const void *)linear_tc_kernel<T, ACC>, smem, ready,
+                           [&] { return cudaLaunchKernelEx(&cfg, linear_tc_kernel<T, ACC>, p, tw, tx, ty); });
 }
 
 template <class T>

@@ -656,11 +656,10 @@ bool gen_layout(const LisArgs &a, GenParams &p, uint32_t &smem)
 template <int NKB, bool MASK, int D>
 cudaError_t gen_launch(const GenParams &p, uint32_t smem, int grid, cudaStream_t st)
 {
-    cudaError_t e = check_smem_fits((const void *)lis_attn_gen_kernel<NKB, MASK, D>, smem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(lis_attn_gen_kernel<NKB, MASK, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    return launch_pdl(lis_attn_gen_kernel<NKB, MASK, D>, dim3(grid), dim3(GTHREADS), smem, st, p);
+    static SmemReady ready;
+    return launch_prepared((const void *)lis_attn_gen_kernel<NKB, MASK, D>, smem, ready, [&] {
+        return launch_pdl(lis_attn_gen_kernel<NKB, MASK, D>, dim3(grid), dim3(GTHREADS), smem, st, p);
+    });
 }
 
 template <int D>

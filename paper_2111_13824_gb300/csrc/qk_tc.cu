@@ -455,11 +455,10 @@ constexpr size_t kQkStaticSmem = sizeof(QkShared) + 64;
 template <bool FOLD, bool BULK>
 cudaError_t qk_launch(const QkParams &p, const CUtensorMap &tm, size_t smem, int grid, cudaStream_t st)
 {
-    cudaError_t e = check_smem_fits((const void *)qk_logits_tc_kernel<FOLD, BULK>, smem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(qk_logits_tc_kernel<FOLD, BULK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    return launch_pdl(qk_logits_tc_kernel<FOLD, BULK>, dim3(grid), dim3(QALL), smem, st, p, tm);
+    static SmemReady ready;
+    return launch_prepared((const void *)qk_logits_tc_kernel<FOLD, BULK>, smem, ready, [&] {
+        return launch_pdl(qk_logits_tc_kernel<FOLD, BULK>, dim3(grid), dim3(QALL), smem, st, p, tm);
+    });
 }
 
 // The logits as a 3-d tensor [BH][L][ld] of bytes for the tensor stores: boxes of 128 x 128 x 1,

@@ -130,12 +130,15 @@ def _p(t):
         raise TypeError("expected a torch.Tensor")
     if not t.is_cuda:
         raise ValueError("libfqvit takes device tensors (got a CPU tensor)")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    """The handle of a stream, by default the current one of the current device."""
+    if stream is not None:
+        return stream.cuda_stream
+    # torch.cuda.current_stream() builds a Stream object around the same handle (3.1 us against 0.2 us a call)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _ld(t: torch.Tensor) -> int:
