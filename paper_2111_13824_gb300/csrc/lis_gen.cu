@@ -89,7 +89,7 @@ struct GenParams {
     int mask_c;  // |mask value| clamped to 1024 (exact: lis_win.cu)
     uint8_t *out8;
     int64_t ld_out8;
-    int n1, n2, zp8;
+    Requant8 rq;
     uint32_t off_c, off_v, off_lg, off_b, off_r;  // shared-memory offsets: control, V ring, logits, bias, regions
 };
 
@@ -505,11 +505,10 @@ __global__ void __launch_bounds__(GTHREADS, 1) lis_attn_gen_kernel(const __grid_
                     uint32_t w[4];
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
-                        w[k] = 0;
+                        int q[4];
 #pragma unroll
-                        for (int u = 0; u < 4; ++u)
-                            w[k] |= requant8(__float2int_rn(__uint_as_float(a[4 * k + u])) - zsum, p.n1, p.n2, p.zp8)
-                                    << (8 * u);
+                        for (int u = 0; u < 4; ++u) q[u] = __float2int_rn(__uint_as_float(a[4 * k + u])) - zsum;
+                        w[k] = requant8x4(q[0], q[1], q[2], q[3], p.rq);
                     }
                     *reinterpret_cast<uint4 *>(p.out8 + row * p.ld_out8 + 16 * c) = make_uint4(w[0], w[1], w[2], w[3]);
                 } else {
@@ -716,9 +715,7 @@ cudaError_t launch_lis_attention_gen(const LisArgs &a, const AttnVArgs &b, cudaS
     p.mask_c = a.mask_value < -1024 ? 1024 : -a.mask_value;
     p.out8 = b.out8;
     p.ld_out8 = b.ld_out8;
-    p.n1 = b.rq_n1;
-    p.n2 = b.rq_n2;
-    p.zp8 = b.rq_zp;
+    p.rq = requant8_of(b.rq_n1, b.rq_n2, b.rq_zp, b.zp_v);
     uint32_t smem;
     if (!gen_layout(a, p, smem)) return cudaErrorInvalidConfiguration;
     const int64_t ntiles = p.pack ? (b.BH * a.L + GM - 1) / GM : b.BH * ((a.L + GM - 1) / GM);

@@ -173,9 +173,9 @@ struct TcParams {
     int L;
     int zp;    // zero point of V (acc = sum_j 2^(15-code) (V - zp))
     IexpC ic;  // Algorithm 1 constants of the scale
-    uint8_t *out8;  // when not null: 8-bit outputs (requant8 with n1, n2, zp8) instead of acc
+    uint8_t *out8;  // when not null: 8-bit outputs instead of acc
     int64_t ld_out8;
-    int n1, n2, zp8;
+    Requant8 rq;
     uint32_t smem;  // dynamic shared memory of the launch
 };
 
@@ -368,11 +368,10 @@ __device__ __forceinline__ void read_out_row(const TcParams &p, uint32_t etl, ui
             uint32_t wq[8];
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
-                wq[c] = 0;
+                int a[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    wq[c] |= requant8(__float2int_rn(__uint_as_float(va[4 * c + k])) - zsum, p.n1, p.n2, p.zp8)
-                             << (8 * k);
+                for (int k = 0; k < 4; ++k) a[k] = __float2int_rn(__uint_as_float(va[4 * c + k])) - zsum;
+                wq[c] = requant8x4(a[0], a[1], a[2], a[3], p.rq);
             }
             uint4 *d8 = reinterpret_cast<uint4 *>(p.out8 + (size_t)grow * p.ld_out8 + 32 * h);
             d8[0] = make_uint4(wq[0], wq[1], wq[2], wq[3]);
@@ -966,7 +965,7 @@ cudaError_t launch_lis_attention_tc(const LisArgs &a, const AttnVArgs &b, cudaSt
     const bool pack = use_pack(a.L);
     const uint32_t smem = tc_smem_bytes(a.L, a.ld_logit, pack);
     TcParams p{a.logits, a.ld_logit, b.v, b.acc, b.BH, a.L, b.zp_v, iexp_consts_host(a.s_logit),
-               b.out8, b.ld_out8, b.rq_n1, b.rq_n2, b.rq_zp, smem};
+               b.out8, b.ld_out8, requant8_of(b.rq_n1, b.rq_n2, b.rq_zp, b.zp_v), smem};
     const int64_t ntiles = pack ? (b.BH * a.L + TM - 1) / TM : b.BH * ((a.L + TM - 1) / TM);
     const int grid = (int)(ntiles < sm_count() ? ntiles : sm_count());
     const bool se = small_iexp(p.ic);

@@ -67,9 +67,9 @@ struct WinParams {
     IexpC ic;
     int ne;  // table entries: distances 0 .. ne - 1
     int ng;  // groups per CTA
-    uint8_t *out8;  // when not null: 8-bit outputs (requant8 with n1, n2, zp8) instead of acc
+    uint8_t *out8;  // when not null: 8-bit outputs instead of acc
     int64_t ld_out8;
-    int n1, n2, zp8;
+    Requant8 rq;
     const uint8_t *region;  // shifted-window mask: region ids [n_windows][L] (MASK variants)
     int n_windows;
     int mask_c;  // |mask value| clamped to 1024 (exact: see the kernel)
@@ -265,12 +265,11 @@ __global__ void __launch_bounds__(WMAXG * 128, 1) lis_attn_win_kernel(WinParams 
             tmem_ld8(tD + 8u * c, va);
             tmem_wait_ld();
             if (ok && p.out8) {  // 8 bytes of 8-bit outputs
-                uint32_t lo = 0, hi = 0;
+                int a[8];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    lo |= requant8(__float2int_rn(__uint_as_float(va[j])) - zsum, p.n1, p.n2, p.zp8) << (8 * j);
-                    hi |= requant8(__float2int_rn(__uint_as_float(va[4 + j])) - zsum, p.n1, p.n2, p.zp8) << (8 * j);
-                }
+                for (int j = 0; j < 8; ++j) a[j] = __float2int_rn(__uint_as_float(va[j])) - zsum;
+                const uint32_t lo = requant8x4(a[0], a[1], a[2], a[3], p.rq);
+                const uint32_t hi = requant8x4(a[4], a[5], a[6], a[7], p.rq);
                 *reinterpret_cast<uint2 *>(p.out8 + ((size_t)bh * L + i) * p.ld_out8 + 8 * c) = make_uint2(lo, hi);
             } else if (ok) {
                 int v8[8];
@@ -577,7 +576,7 @@ cudaError_t launch_lis_attention_win(const LisArgs &a, const AttnVArgs &b, cudaS
 {
     const bool bias = a.bias != nullptr;
     WinParams p{a.logits, a.ld_logit, b.v, b.ld_v, b.acc, b.ld_acc, a.bias, a.heads, a.window, b.BH, a.L, b.zp_v,
-                iexp_consts_host(a.s_logit), 0, 0, b.out8, b.ld_out8, b.rq_n1, b.rq_n2, b.rq_zp,
+                iexp_consts_host(a.s_logit), 0, 0, b.out8, b.ld_out8, requant8_of(b.rq_n1, b.rq_n2, b.rq_zp, b.zp_v),
                 a.region, a.n_windows, a.mask_value < -1024 ? 1024 : -a.mask_value};
     const int mwin = a.region ? a.n_windows : 0;
     p.ne = win_table_entries(p.ic, bias);
