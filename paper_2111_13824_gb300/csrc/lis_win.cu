@@ -31,6 +31,10 @@
 // address.  Distances past 15 |q_ln2| all give e(15 |q_ln2|) (the clamp of
 // Algorithm 1), so d is clamped to ne - 1.
 //
+// Issue-bound: about 40 instructions per key.  Swin-S stage 1 with bias and mask (12288
+// heads of 49 keys) 67.8 us -> 58.9: the code from exponents (code_ops), 13 words of keys
+// instead of 16, no mask arithmetic in the windows of one region.
+//
 // Every wait is bounded (two seconds), after which the group stops, records a
 // timeout status and the kernel drains what it issued.
 #include "fqvit_internal.cuh"
@@ -94,30 +98,20 @@ __device__ __forceinline__ uint32_t lut_off(uint32_t dpair, uint32_t lane4)
     return prmt(dpair, lane4, SEL);
 }
 
-// fp16 exponent field (30 - code) of the operand 2^(15-code), as operand_exp_f with D_k read
-// from a table (dk[k] = D_k for k = 1 .. 63; k <= 43 since 2S < 2^43 and e >= 1)
-__device__ __forceinline__ uint32_t operand_exp_tab(float ef, int G, float hi, float lo, const float *dk)
-{
-    const int k = (G - __float_as_int(ef)) >> 23;
-    const float t = __fmaf_rn(ef, dk[k], -hi);
-    uint32_t le;  // 0xFFFFFFFF when e D_k <= 2S
-    asm("set.le.u32.f32 %0, %1, %2;" : "=r"(le) : "f"(t), "f"(lo));
-    return (uint32_t)max(31 - k + (int)le, 15);
-}
-
-// NQ: 16-key chunks of a row (L in 16 (NQ - 1) + 1 .. 16 NQ).  MASK (with BIAS): the shifted-window
-// mask.  Logits then sit in the 16-bit lanes as v = q + bias + 1280 - (masked ? m_c : 0) with m_c the
+// NW: words of four keys of a row, ceil(L / 4) <= NW (13: exactly, the 49 keys of a 7 x 7 window; with whole
+// 16-key chunks a fourth of their pairs were padding).  MASK (with BIAS): the shifted-window mask; windows of
+// one region (all but the last row and column of the map) skip its arithmetic.  Logits then sit in the 16-bit lanes as v = q + bias + 1280 - (masked ? m_c : 0) with m_c the
 // mask magnitude clamped to 1024: a key masked by more still lands below every unmasked key (the
 // query's own key is never masked, v >= 1024) at a distance above 510 >= the table's last entry,
 // which is the clamp 15 |q_ln2| of Algorithm 1 (the launch requires 15 |q_ln2| <= 510), so its
 // i-exp value and the row maximum are those of the true mask.
-template <int D, bool BIAS, bool SMALL_E, int NQ, bool MASK>
+template <int D, bool BIAS, bool SMALL_E, int NW, bool MASK>
 __global__ void __launch_bounds__(WMAXG * 128, 1) lis_attn_win_kernel(WinParams p)
 {
+    constexpr int NQ = (NW + 3) / 4;  // 16-key chunks
     extern __shared__ __align__(16) unsigned char dsm_raw[];
     __shared__ WinShared sh;
     __shared__ uint32_t e_tmp[512];
-    __shared__ float dk[64];
     __shared__ int koff[64], qbase[64];  // relative-position offsets (bias only)
     // the table first, at the fixed start of dynamic shared memory (lookups add no base), then
     // B (1024-byte aligned for the 128-byte swizzle) and the bias rows
@@ -126,6 +120,7 @@ __global__ void __launch_bounds__(WMAXG * 128, 1) lis_attn_win_kernel(WinParams 
     unsigned char *Bs_all = dsm_raw + bs_off + ((1024u - ((sa(dsm_raw) + bs_off) & 1023u)) & 1023u);  // ng x 16 KB
     unsigned char *BR = Bs_all + p.ng * WB_BYTES;                             // heads x L x 64 B
     unsigned char *RG = BR + (BIAS ? (size_t)p.heads * p.L * WBIAS_ROW : 0);  // n_windows x 64 B region ids
+    unsigned char *RU = RG + (MASK ? p.n_windows * 64 : 0);                    // n_windows: more than one region
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = tid >> 7, r = tid & 127;
@@ -148,11 +143,9 @@ __global__ void __launch_bounds__(WMAXG * 128, 1) lis_attn_win_kernel(WinParams 
                      "r"(win_tmem_cols(p.ng)));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
-    // set-up, phase 1: i-exp values, the D_k table, the raw bias table (into the B area, free
+    // set-up, phase 1: i-exp values, the raw bias table (into the B area, free
     // until phase 3) and the index offsets of the relative positions
     for (int d = tid; d < p.ne; d += blockDim.x) e_tmp[d] = iexp_neg(d, p.ic);
-    for (int k = tid; k < 64; k += blockDim.x)  // D_1 = 3, D_k = 3 2^(k-1) - 1 (exact up to k = 24)
-        dk[k] = k <= 1 ? 3.0f : __fsub_rn(__int_as_float(((k + 127) << 23) | 0x400000), 1.0f);
     const int nb = 2 * p.window - 1;
     pdl_wait();  // the first access to global memory follows
     if (BIAS) {
@@ -197,6 +190,13 @@ __global__ void __launch_bounds__(WMAXG * 128, 1) lis_attn_win_kernel(WinParams 
             const int wdx = x >> 6, j = x & 63;
             RG[x] = j < L ? p.region[(size_t)wdx * L + j] : 0;
         }
+    if (MASK)
+        for (int w = tid; w < p.n_windows; w += blockDim.x) {
+            const uint8_t *r = p.region + (size_t)w * L;
+            int many = 0;
+            for (int j = 1; j < L; ++j) many |= r[j] ^ r[0];
+            RU[w] = many ? 1 : 0;
+        }
     // phase 3: B of every group: zeros, and (d = 32) fp16 1 in column 32 of every key row below L
     for (int x = tid; x < p.ng * WB_BYTES / 16; x += blockDim.x) {
         const int kk = (x >> 3) & 127, pos = x & 7, ci = pos ^ (kk & 7);
@@ -219,7 +219,8 @@ __global__ void __launch_bounds__(WMAXG * 128, 1) lis_attn_win_kernel(WinParams 
     const uint32_t tA = tD + 64u;
     unsigned char *Bg = Bs_all + g * WB_BYTES;
     const uint32_t lane4 = (uint32_t)lane << 2;
-    const int nw = (L + 3) >> 2;   // words that hold keys (all but the last chunk's are full)
+    const int nw = NW == 13 ? 13 : (L + 3) >> 2;   // words that hold keys (all but the last chunk's are full)
+    const float e0 = __uint2float_rn(e_tmp[0]);
     uint32_t cm[4];                // byte masks of the last chunk's words: keys below L
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -296,54 +297,51 @@ __global__ void __launch_bounds__(WMAXG * 128, 1) lis_attn_win_kernel(WinParams 
         const int bh = 2 * t + h;
         const bool valid = bh < BH && i < L;
         // ---- q + 128 per byte, keys past L zeroed (only the last chunk has any)
-        uint32_t u[4 * NQ];
+        uint32_t u[NW];
 #pragma unroll
-        for (int c = 0; c < NQ; ++c) {
-            const uint32_t ww[4] = {w[c].x, w[c].y, w[c].z, w[c].w};
-#pragma unroll
-            for (int k = 0; k < 4; ++k) u[4 * c + k] = (ww[k] ^ 0x80808080u) & (c == NQ - 1 ? cm[k] : 0xFFFFFFFFu);
+        for (int j = 0; j < NW; ++j) {
+            const uint32_t ww[4] = {w[j >> 2].x, w[j >> 2].y, w[j >> 2].z, w[j >> 2].w};
+            u[j] = (ww[j & 3] ^ 0x80808080u) & (j >= 4 * (NQ - 1) ? cm[j & 3] : 0xFFFFFFFFu);
         }
         // ---- pairs of 16-bit lanes v = q + bias + 256 (0 for keys past L):
         //      vp[2j] holds keys (4j, 4j+2), vp[2j+1] keys (4j+1, 4j+3)
-        uint32_t vp[8 * NQ];
-        if (MASK) {
+        uint32_t vp[2 * NW];
+        if (BIAS) {
             const unsigned char *br = BR + ((size_t)hh * L + qi) * WBIAS_ROW;
-            const unsigned char *rg = RG + (size_t)((bh / p.heads) % p.n_windows) * 64;
-            const uint32_t rib = (uint32_t)rg[qi] * 0x01010101u;
+            const int wdx = MASK ? (bh / p.heads) % p.n_windows : 0;
 #pragma unroll
             for (int c = 0; c < NQ; ++c) {
                 const uint4 b4 = *reinterpret_cast<const uint4 *>(br + 16 * (c ^ sw));
-                const uint4 r4 = *reinterpret_cast<const uint4 *>(rg + 16 * c);
                 const uint32_t bb[4] = {b4.x, b4.y, b4.z, b4.w};
-                const uint32_t rr[4] = {r4.x, r4.y, r4.z, r4.w};
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
+                for (int k = 0; k < 4 && 4 * c + k < NW; ++k) {
                     const int j = 4 * c + k;
-                    // byte nonzero: the key's region differs from the query's (keys past L: never)
-                    const uint32_t x = (rr[k] ^ rib) & (c == NQ - 1 ? cm[k] : 0xFFFFFFFFu);
-                    const uint32_t me = ((prmt(x, 0u, 0x4240u) + 0x7FFF7FFFu) >> 15) & 0x00010001u;
-                    const uint32_t mo = ((prmt(x, 0u, 0x4341u) + 0x7FFF7FFFu) >> 15) & 0x00010001u;
-                    vp[2 * j] = prmt(u[j], 0u, 0x4240u) + prmt(bb[k], 0u, 0x4240u) + 0x04000400u - me * (uint32_t)p.mask_c;
-                    vp[2 * j + 1] =
-                        prmt(u[j], 0u, 0x4341u) + prmt(bb[k], 0u, 0x4341u) + 0x04000400u - mo * (uint32_t)p.mask_c;
+                    vp[2 * j] = prmt(u[j], 0u, 0x4240u) + prmt(bb[k], 0u, 0x4240u) + (MASK ? 0x04000400u : 0u);
+                    vp[2 * j + 1] = prmt(u[j], 0u, 0x4341u) + prmt(bb[k], 0u, 0x4341u) + (MASK ? 0x04000400u : 0u);
                 }
             }
-        } else if (BIAS) {
-            const unsigned char *br = BR + ((size_t)hh * L + qi) * WBIAS_ROW;
+            if (MASK && RU[wdx]) {  // (uniform over the warp: its rows lie in one window)
+                const unsigned char *rg = RG + wdx * 64;
+                const uint32_t rib = (uint32_t)rg[qi] * 0x01010101u;
 #pragma unroll
-            for (int c = 0; c < NQ; ++c) {
-                const uint4 b4 = *reinterpret_cast<const uint4 *>(br + 16 * (c ^ sw));
-                const uint32_t bb[4] = {b4.x, b4.y, b4.z, b4.w};
+                for (int c = 0; c < NQ; ++c) {
+                    const uint4 r4 = *reinterpret_cast<const uint4 *>(rg + 16 * c);
+                    const uint32_t rr[4] = {r4.x, r4.y, r4.z, r4.w};
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int j = 4 * c + k;
-                    vp[2 * j] = prmt(u[j], 0u, 0x4240u) + prmt(bb[k], 0u, 0x4240u);
-                    vp[2 * j + 1] = prmt(u[j], 0u, 0x4341u) + prmt(bb[k], 0u, 0x4341u);
+                    for (int k = 0; k < 4 && 4 * c + k < NW; ++k) {
+                        const int j = 4 * c + k;
+                        // byte nonzero: the key's region differs from the query's (keys past L: never)
+                        const uint32_t x = (rr[k] ^ rib) & (c == NQ - 1 ? cm[k] : 0xFFFFFFFFu);
+                        const uint32_t me = ((prmt(x, 0u, 0x4240u) + 0x7FFF7FFFu) >> 15) & 0x00010001u;
+                        const uint32_t mo = ((prmt(x, 0u, 0x4341u) + 0x7FFF7FFFu) >> 15) & 0x00010001u;
+                        vp[2 * j] -= me * (uint32_t)p.mask_c;
+                        vp[2 * j + 1] -= mo * (uint32_t)p.mask_c;
+                    }
                 }
             }
         } else {
 #pragma unroll
-            for (int j = 0; j < 4 * NQ; ++j) {
+            for (int j = 0; j < NW; ++j) {
                 vp[2 * j] = prmt(u[j], 0u, 0x4240u);
                 vp[2 * j + 1] = prmt(u[j], 0u, 0x4341u);
             }
@@ -351,11 +349,11 @@ __global__ void __launch_bounds__(WMAXG * 128, 1) lis_attn_win_kernel(WinParams 
         // ---- row maximum (keys past L are 0), then distances d = max - v clamped to the table
         uint32_t mx = vmax16x2u(vp[0], vp[1]);
 #pragma unroll
-        for (int k = 2; k < 8 * NQ; k += 2) mx = vmax16x2u(mx, vmax16x2u(vp[k], vp[k + 1]));
+        for (int k = 2; k < 2 * NW; k += 2) mx = vmax16x2u(mx, vmax16x2u(vp[k], vp[k + 1]));
         const uint32_t m = max(mx & 0xFFFFu, mx >> 16);
         const uint32_t m2 = m * 0x10001u;
 #pragma unroll
-        for (int k = 0; k < 8 * NQ; ++k) vp[k] = vmin16x2u(m2 - vp[k], cap2);
+        for (int k = 0; k < 2 * NW; ++k) vp[k] = vmin16x2u(m2 - vp[k], cap2);
         // ---- i-exp row sum over the words that hold keys (padding keys of the last word have
         //      d = max; they are taken out below)
         unsigned long long S = 0;
@@ -365,8 +363,8 @@ __global__ void __launch_bounds__(WMAXG * 128, 1) lis_attn_win_kernel(WinParams 
             unsigned long long a64 = 0;
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
-                if (c < NQ - 1 || 4 * c + (k >> 1) < nw) {
-                    const uint32_t dp = vp[8 * c + k];
+                if (4 * c + (k >> 1) < NW && (c < NQ - 1 || 4 * c + (k >> 1) < nw)) {
+                    const uint32_t dp = vp[8 * c + k < 2 * NW ? 8 * c + k : 0];
                     const uint32_t e0 = *reinterpret_cast<const uint32_t *>(LUTB + lut_off<0x5104u>(dp, lane4));
                     const uint32_t e1 = *reinterpret_cast<const uint32_t *>(LUTB + lut_off<0x5324u>(dp, lane4));
                     if (SMALL_E)
@@ -383,7 +381,8 @@ __global__ void __launch_bounds__(WMAXG * 128, 1) lis_attn_win_kernel(WinParams 
             const uint32_t epad = *reinterpret_cast<const uint32_t *>(LUTB + ((dm << 8) | lane4));
             S -= (unsigned long long)(4 * nw - L) * epad;
         }
-        const RowSum rs = split_2s(S);
+        const CodeRow rs = code_row(S, e0);
+        const bool any_fix = __any_sync(0xffffffffu, rs.fix != 0);
         // V key row i of this slot (used after the operands: its latency hides behind them)
         uint4 vv[D / 16];
         {
@@ -409,23 +408,28 @@ __global__ void __launch_bounds__(WMAXG * 128, 1) lis_attn_win_kernel(WinParams 
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const int j = 4 * c + k;
-                if (c == NQ - 1 && j >= nw) {
+                if (j >= NW || (c == NQ - 1 && j >= nw)) {
                     o[2 * k] = o[2 * k + 1] = 0u;
                     continue;
                 }
-                const uint32_t de = vp[2 * j], dod = vp[2 * j + 1];
+                const uint32_t de = vp[j < NW ? 2 * j : 0], dod = vp[j < NW ? 2 * j + 1 : 0];
                 const float f0 = *reinterpret_cast<const float *>(LUTB + 128 + lut_off<0x5104u>(de, lane4));
                 const float f2 = *reinterpret_cast<const float *>(LUTB + 128 + lut_off<0x5324u>(de, lane4));
                 const float f1 = *reinterpret_cast<const float *>(LUTB + 128 + lut_off<0x5104u>(dod, lane4));
                 const float f3 = *reinterpret_cast<const float *>(LUTB + 128 + lut_off<0x5324u>(dod, lane4));
-                const uint32_t E0 = operand_exp_tab(f0, rs.hibits, rs.hi, rs.lo, dk);
-                const uint32_t E1 = operand_exp_tab(f1, rs.hibits, rs.hi, rs.lo, dk);
-                const uint32_t E2 = operand_exp_tab(f2, rs.hibits, rs.hi, rs.lo, dk);
-                const uint32_t E3 = operand_exp_tab(f3, rs.hibits, rs.hi, rs.lo, dk);
-                o[2 * k] = (E0 << 10) | (E1 << 26);
-                o[2 * k + 1] = (E2 << 10) | (E3 << 26);
+                o[2 * k] = code_ops(f0, f1, rs);
+                o[2 * k + 1] = code_ops(f2, f3, rs);
+                if (any_fix) {  // the key at distance 0, where 3 e > 2S
+                    const uint32_t ze = 0x00010001u - vmin16x2u(de, 0x00010001u);
+                    const uint32_t zo = 0x00010001u - vmin16x2u(dod, 0x00010001u);
+                    o[2 * k] += prmt(ze, zo, 0x5410u) * rs.fix;
+                    o[2 * k + 1] += prmt(ze, zo, 0x7632u) * rs.fix;
+                }
             }
-            tmem_st8(tA + 32u * (uint32_t)h + 8u * c, o);
+            if (4 * c + 1 == NW)  // one word: the columns behind it keep the zeros of the start
+                tmem_st2(tA + 32u * (uint32_t)h + 8u * c, o[0], o[1]);
+            else
+                tmem_st8(tA + 32u * (uint32_t)h + 8u * c, o);
         }
         // ---- V key row i of this slot -> fp16 B (row 64 h + i, chunk ci at ci ^ (row & 7))
         if (valid) {
@@ -487,13 +491,13 @@ __global__ void __launch_bounds__(WMAXG * 128, 1) lis_attn_win_kernel(WinParams 
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(win_tmem_cols(p.ng)));
 }
 
-constexpr size_t kWinStaticSmem = 512 * 4 + 64 * 4 * 3 + sizeof(WinShared) + 256;
+constexpr size_t kWinStaticSmem = 512 * 4 + 64 * 4 * 2 + sizeof(WinShared) + 256;
 constexpr size_t kSmemLimit = 232448;
 
 size_t win_smem_bytes(int ng, int ne, int heads, int L, bool bias, int mask_windows)
 {
     return 1024 + (size_t)ng * WB_BYTES + (size_t)ne * 256 + (bias ? (size_t)heads * L * WBIAS_ROW : 0) +
-           (size_t)mask_windows * 64;
+           (size_t)mask_windows * 65;
 }
 
 // table entries: distances up to 255 (510 with a bias), and none past the clamp 15 |q_ln2|
@@ -518,23 +522,25 @@ int win_groups(int ne, int heads, int L, int window, bool bias, int mask_windows
 
 bool small_iexp_w(const IexpC &c) { return ((double)c.q_b * c.q_b + c.q_c) * 32768.0 < 268435456.0; }
 
-template <int D, bool BIAS, bool SMALL_E, int NQ, bool MASK>
+template <int D, bool BIAS, bool SMALL_E, int NW, bool MASK>
 cudaError_t win_launch_q(const WinParams &p, size_t smem, int grid, cudaStream_t st)
 {
     static SmemReady ready;
-    return launch_prepared((const void *)lis_attn_win_kernel<D, BIAS, SMALL_E, NQ, MASK>, smem, ready, [&] {
-        return launch_pdl(lis_attn_win_kernel<D, BIAS, SMALL_E, NQ, MASK>, dim3(grid), dim3(128 * p.ng), smem, st, p);
+    return launch_prepared((const void *)lis_attn_win_kernel<D, BIAS, SMALL_E, NW, MASK>, smem, ready, [&] {
+        return launch_pdl(lis_attn_win_kernel<D, BIAS, SMALL_E, NW, MASK>, dim3(grid), dim3(128 * p.ng), smem, st, p);
     });
 }
 
 template <int D, bool BIAS, bool SMALL_E, bool MASK>
 cudaError_t win_launch(const WinParams &p, size_t smem, int grid, cudaStream_t st)
 {
-    switch ((p.L + 15) >> 4) {
-    case 1: return win_launch_q<D, BIAS, SMALL_E, 1, MASK>(p, smem, grid, st);
-    case 2: return win_launch_q<D, BIAS, SMALL_E, 2, MASK>(p, smem, grid, st);
-    case 3: return win_launch_q<D, BIAS, SMALL_E, 3, MASK>(p, smem, grid, st);
-    default: return win_launch_q<D, BIAS, SMALL_E, 4, MASK>(p, smem, grid, st);
+    const int nw = (p.L + 3) >> 2;
+    if (nw == 13) return win_launch_q<D, BIAS, SMALL_E, 13, MASK>(p, smem, grid, st);
+    switch ((nw + 3) >> 2) {
+    case 1: return win_launch_q<D, BIAS, SMALL_E, 4, MASK>(p, smem, grid, st);
+    case 2: return win_launch_q<D, BIAS, SMALL_E, 8, MASK>(p, smem, grid, st);
+    case 3: return win_launch_q<D, BIAS, SMALL_E, 12, MASK>(p, smem, grid, st);
+    default: return win_launch_q<D, BIAS, SMALL_E, 16, MASK>(p, smem, grid, st);
     }
 }
 

@@ -189,6 +189,53 @@ __device__ __forceinline__ RowSum split_2s(unsigned long long S)
     return rs;
 }
 
+// ---- The code of a key from exponents alone.  For k >= 2 the test e D_k <= 2S (lis.cu) reads
+// 2S + e >= 3 2^(k-1) e, so code = floor(log2((2S + e) / (3e/2))): the difference of two fp32 bit patterns,
+// its low 23 bits comparing the mantissas.  3e/2 is exact (e has at most 16 significant bits), and 2S + e
+// rounded toward zero stays on the same side of every 3 2^(k-1) e, which is representable.  With
+// 2S = hi + lo (hi rounded toward zero, lo exact) it is RZ(hi + RZ(lo + e)): RZ(lo + e) is the largest
+// multiple of its own last place below lo + e, and the last place of the sum is no finer.  For k = 1
+// (D_1 = 3, not 2) the difference says 1 where the code is 0, for the one key with 3e > 2S that a row can
+// have, its maximum (CodeRow::fix).  6 operations a key where the D_k test takes 10.
+struct CodeRow {
+    float hi, lo;
+    uint32_t fix;  // 0x0400, to be added to the operand of the maximum when 3 e(0) > 2S, else 0
+};
+
+// e0: the i-exp value of the maximum, fp32
+__device__ __forceinline__ CodeRow code_row(unsigned long long S, float e0)
+{
+    const unsigned long long s2 = 2ull * S;
+    CodeRow r;
+    if (s2 < (1ull << 24)) {
+        r.hi = __uint2float_rn((uint32_t)s2);
+        r.lo = 0.0f;
+    } else {
+        const int p = 63 - __clzll((long long)s2), sh = p - 23;  // p = 24 .. 42
+        r.hi = __int_as_float(((127 + p) << 23) | ((int)(s2 >> sh) & 0x7FFFFF));
+        r.lo = __uint2float_rn((uint32_t)s2 & ((1u << sh) - 1u));  // below 2^19
+    }
+    r.fix = __fmul_rn(3.0f, e0) > r.hi ? 0x0400u : 0u;  // 3 e0 is representable: 3 e0 > hi says 3 e0 > 2S
+    return r;
+}
+
+// a float in [2^(15 - code), 2^(16 - code)) of an i-exp value (before the fix, code not clipped to 15)
+__device__ __forceinline__ float code_pow2(float ef, const CodeRow &r)
+{
+    const float A = __fadd_rz(r.hi, __fadd_rz(r.lo, ef)), g = __fmul_rn(1.5f, ef);
+    return __int_as_float(__float_as_int(g) - __float_as_int(A) + ((143 << 23) - 1));
+}
+
+// the fp16 operands 2^(15 - code) of two keys (low, high half), codes clipped to 15
+__device__ __forceinline__ uint32_t code_ops(float f0, float f1, const CodeRow &r)
+{
+    uint32_t d;
+    asm("cvt.rz.f16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(code_pow2(f1, r)), "f"(code_pow2(f0, r)));
+    d &= 0x7C007C00u;
+    asm("max.u16x2 %0, %0, %1;" : "+r"(d) : "r"(0x3C003C00u));
+    return d;
+}
+
 // mbar_wait with one verdict for the whole warp (the callers go on to
 // warp-collective tcgen05 instructions)
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t *b, uint32_t parity, volatile int *abort_flag)
