@@ -19,8 +19,8 @@
 // Roles (22 warps):
 //   warps 0-15, four threads per row (warp 4 q + r / 32, lane r % 32; part q takes keys
 //     64 kb + 16 q .. of every 64-key block, or 4 keys of a last block of at most
-//     16): row maximum, i-exp row sum, then each key's code by the exact test
-//     e D_k <= 2S (lis.cu), the operands straight into tensor memory.  Only the
+//     16): row maximum, i-exp row sum, then each key's code (code_ops,
+//     tc_common.cuh), the operands straight into tensor memory.  Only the
 //     four warps of 32 rows meet (two named barriers per tile), so the four
 //     groups drift apart and one's lookups overlap another's reductions.
 //     Without a bias the logits are read again from shared memory in each of
@@ -123,6 +123,27 @@ __device__ __forceinline__ GTile gen_tile(const GenParams &p, int64_t t, int tpb
     return ti;
 }
 
+// the tile after ti (a step of GM <= L rows crosses at most one head boundary)
+__device__ __forceinline__ GTile gen_next(const GenParams &p, GTile ti)
+{
+    if (p.pack) {
+        ti.g0 += GM;
+        if (ti.g0 >= (int64_t)(ti.h0 + 1) * p.L) ++ti.h0;
+        ti.rows = (int)min((int64_t)GM, p.BH * p.L - ti.g0);
+        ti.nsplit = (int)min((int64_t)ti.rows, (int64_t)(ti.h0 + 1) * p.L - ti.g0);
+    } else {
+        int r0 = (int)(ti.g0 - (int64_t)ti.h0 * p.L) + GM;
+        if (r0 >= p.L) {
+            ++ti.h0;
+            r0 = 0;
+        }
+        ti.g0 = (int64_t)ti.h0 * p.L + r0;
+        ti.rows = min(GM, p.L - r0);
+        ti.nsplit = ti.rows;
+    }
+    return ti;
+}
+
 __device__ __forceinline__ uint32_t ldu32(const unsigned char *p) { return *reinterpret_cast<const uint32_t *>(p); }
 __device__ __forceinline__ float ldf32(const unsigned char *p) { return *reinterpret_cast<const float *>(p); }
 
@@ -136,13 +157,6 @@ template <int J>
 __device__ __forceinline__ uint32_t line_h(uint32_t w, uint32_t off)
 {
     return prmt(w, off, J == 0 ? 0x7104u : 0x7324u);  // off[0], half's low byte, its high byte, 0
-}
-
-// the fp16 pair of the operands of two keys (fp32 i-exp values f0, f1)
-__device__ __forceinline__ uint32_t op_pair(float f0, float f1, const RowSum &rs)
-{
-    const uint32_t a = operand_exp_f(f0, rs.hibits, rs.hi, rs.lo), b = operand_exp_f(f1, rs.hibits, rs.hi, rs.lo);
-    return (a << 10) | (b << 26);
 }
 
 // NKB: 64-key blocks of a biased row (1 .. 4), 0 without a bias (any length, logits re-read)
@@ -166,6 +180,7 @@ __global__ void __launch_bounds__(GTHREADS, 1) lis_attn_gen_kernel(const __grid_
     int *qbase = koff + 64 * NKB;                              // [64 NKB]
     unsigned char *BT = reinterpret_cast<unsigned char *>(qbase + 64 * NKB);  // [heads][nb2], bias + 128
     unsigned char *RG = dsm + p.off_r;                         // [n_windows][Lp]
+    unsigned char *RU = RG + p.n_windows * Lp;                 // [n_windows]: more than one region
     pdl_release();
     if ((sa(dsm) & 1023u) != 0) {  // the swizzled V blocks: reported (FQVIT_ERR_UNSUPPORTED) instead of run
         if (tid == 0) atomicCAS(&g_status, 0, 2);
@@ -224,6 +239,13 @@ __global__ void __launch_bounds__(GTHREADS, 1) lis_attn_gen_kernel(const __grid_
             const int w = x / Lp, j = x - w * Lp;
             RG[x] = j < L ? p.region[(size_t)w * L + j] : 0;
         }
+    if (MASK)
+        for (int w = tid; w < p.n_windows; w += GTHREADS) {
+            const uint8_t *rp = p.region + (size_t)w * L;
+            int many = 0;
+            for (int j = 1; j < L; ++j) many |= rp[j] ^ rp[0];
+            RU[w] = many ? 1 : 0;
+        }
     fence_async_smem();  // ONES and the V blocks are read by the MMAs
     tc_fence_before();
     __syncthreads();
@@ -234,12 +256,14 @@ __global__ void __launch_bounds__(GTHREADS, 1) lis_attn_gen_kernel(const __grid_
     const int64_t ntiles = p.pack ? (p.BH * L + GM - 1) / GM : p.BH * tpb;
     const int64_t t_begin = (int64_t)blockIdx.x * ntiles / gridDim.x;
     const int n = (int)((int64_t)(blockIdx.x + 1) * ntiles / gridDim.x - t_begin);
+    GTile ti = gen_tile(p, t_begin, tpb);
 
     if (warp < GSOFT_WARPS) {
         const int k4 = warp & 3, q = warp >> 2, r = 32 * k4 + lane;
         const uint32_t off = 4u * (uint32_t)lane;
         const uint32_t tA = tmem + G_TA + ((uint32_t)(32 * k4) << 16);
         const uint32_t cap2 = (uint32_t)(p.ne - 1) * 0x10001u;
+        const float e0 = ldf32(dsm + 128);
         // the last block holds R = 1 .. 64 keys; with R <= 16 each part takes 4 of them (see above)
         const int R = L - (nkb - 1) * 64;
         const bool quarter = R <= 16;
@@ -267,8 +291,7 @@ __global__ void __launch_bounds__(GTHREADS, 1) lis_attn_gen_kernel(const __grid_
             asm volatile("bar.sync %0, 128;" ::"r"(1 + k4) : "memory");
         };
         uint32_t ps = 0, pph = 1;  // operand ring (the first pass over it waits for nothing)
-        for (int it = 0; it < n; ++it) {
-            const GTile ti = gen_tile(p, t_begin + it, tpb);
+        for (int it = 0; it < n; ++it, ti = gen_next(p, ti)) {
             const int lb = p.nlg == 2 ? it & 1 : 0;
             const uint32_t lph = (uint32_t)(p.nlg == 2 ? it >> 1 : it) & 1u;
             const unsigned char *lr = LG + (size_t)lb * GM * p.ld + (size_t)r * p.ld;
@@ -286,7 +309,9 @@ __global__ void __launch_bounds__(GTHREADS, 1) lis_attn_gen_kernel(const __grid_
                 const int bh = r < ti.nsplit || ti.nsplit == ti.rows ? ti.h0 : ti.h0 + 1;
                 const int i = min((int)(g - (int64_t)bh * L), L - 1);
                 const unsigned char *bt = BT + (bh % p.heads) * nb2 + qbase[i];
-                const unsigned char *rg = RG + (MASK ? (size_t)((bh / p.heads) % p.n_windows) * Lp : 0);
+                const int wdx = MASK ? (bh / p.heads) % p.n_windows : 0;
+                const unsigned char *rg = RG + wdx * Lp;
+                const bool masked = MASK && __any_sync(0xffffffffu, RU[wdx] != 0);  // some row's window has regions
                 const uint32_t rib = MASK ? (uint32_t)rg[i] * 0x01010101u : 0u;
                 uint32_t mx = 0;
                 auto word = [&](uint32_t w, int key, uint32_t rw, uint32_t &pe, uint32_t &po) {
@@ -296,11 +321,15 @@ __global__ void __launch_bounds__(GTHREADS, 1) lis_attn_gen_kernel(const __grid_
                     pe = prmt(u, 0u, 0x4240u) + (b0 | (b2 << 16));
                     po = prmt(u, 0u, 0x4341u) + (b1 | (b3 << 16));
                     if (MASK) {
-                        const uint32_t x = rw ^ rib;  // byte nonzero: the key's region differs
-                        const uint32_t me = ((prmt(x, 0u, 0x4240u) + 0x7FFF7FFFu) >> 15) & 0x00010001u;
-                        const uint32_t mo = ((prmt(x, 0u, 0x4341u) + 0x7FFF7FFFu) >> 15) & 0x00010001u;
-                        pe = pe + 0x04000400u - me * (uint32_t)p.mask_c;
-                        po = po + 0x04000400u - mo * (uint32_t)p.mask_c;
+                        pe += 0x04000400u;
+                        po += 0x04000400u;
+                        if (masked) {
+                            const uint32_t x = rw ^ rib;  // byte nonzero: the key's region differs
+                            const uint32_t me = ((prmt(x, 0u, 0x4240u) + 0x7FFF7FFFu) >> 15) & 0x00010001u;
+                            const uint32_t mo = ((prmt(x, 0u, 0x4341u) + 0x7FFF7FFFu) >> 15) & 0x00010001u;
+                            pe -= me * (uint32_t)p.mask_c;
+                            po -= mo * (uint32_t)p.mask_c;
+                        }
                     }
                 };
 #pragma unroll
@@ -390,15 +419,27 @@ __global__ void __launch_bounds__(GTHREADS, 1) lis_attn_gen_kernel(const __grid_
             red_sum[q * GM + r] = S;
             group_bar();
             S = red_sum[r] + red_sum[GM + r] + red_sum[2 * GM + r] + red_sum[3 * GM + r];
-            const RowSum rs = split_2s(S);
+            const CodeRow rs = code_row(S, e0);
+            const bool any_fix = __any_sync(0xffffffffu, rs.fix != 0);
             // ---- operands, block after block, into the ring
             auto ops4 = [&](uint32_t w, uint32_t &o0, uint32_t &o1) {  // a word of four distance bytes
-                o0 = op_pair(ldf32(dsm + 128 + line_b<0>(w, off)), ldf32(dsm + 128 + line_b<1>(w, off)), rs);
-                o1 = op_pair(ldf32(dsm + 128 + line_b<2>(w, off)), ldf32(dsm + 128 + line_b<3>(w, off)), rs);
+                o0 = code_ops(ldf32(dsm + 128 + line_b<0>(w, off)), ldf32(dsm + 128 + line_b<1>(w, off)), rs);
+                o1 = code_ops(ldf32(dsm + 128 + line_b<2>(w, off)), ldf32(dsm + 128 + line_b<3>(w, off)), rs);
+                if (any_fix) {  // the key at distance 0, where 3 e > 2S
+                    const uint32_t z = (~(((w & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | w) >> 7) & 0x01010101u;
+                    o0 += prmt(z, 0u, 0x4140u) * rs.fix;
+                    o1 += prmt(z, 0u, 0x4342u) * rs.fix;
+                }
             };
             auto ops4h = [&](uint32_t pe, uint32_t po, uint32_t &o0, uint32_t &o1) {  // two pairs of 16-bit distances
-                o0 = op_pair(ldf32(dsm + 128 + line_h<0>(pe, off)), ldf32(dsm + 128 + line_h<0>(po, off)), rs);
-                o1 = op_pair(ldf32(dsm + 128 + line_h<1>(pe, off)), ldf32(dsm + 128 + line_h<1>(po, off)), rs);
+                o0 = code_ops(ldf32(dsm + 128 + line_h<0>(pe, off)), ldf32(dsm + 128 + line_h<0>(po, off)), rs);
+                o1 = code_ops(ldf32(dsm + 128 + line_h<1>(pe, off)), ldf32(dsm + 128 + line_h<1>(po, off)), rs);
+                if (any_fix) {
+                    const uint32_t ze = 0x00010001u - vmin16x2u(pe, 0x00010001u);
+                    const uint32_t zo = 0x00010001u - vmin16x2u(po, 0x00010001u);
+                    o0 += prmt(ze, zo, 0x5410u) * rs.fix;
+                    o1 += prmt(ze, zo, 0x7632u) * rs.fix;
+                }
             };
             auto block_out = [&](bool last, uint32_t (&o)[8]) {
                 mbar_wait_warp(&sh.pfree[ps], pph, abort_flag);  // the MMAs of the slot's previous block are done
@@ -526,8 +567,7 @@ __global__ void __launch_bounds__(GTHREADS, 1) lis_attn_gen_kernel(const __grid_
             if (lane == 0) mbar_arrive(&sh.dfree[par]);
         };
         GTile prev{};
-        for (int it = 0; it < n; ++it) {
-            const GTile ti = gen_tile(p, t_begin + it, tpb);
+        for (int it = 0; it < n; ++it, ti = gen_next(p, ti)) {
             if (it > 0) read_out(prev, (it - 1) & 1, (uint32_t)((it - 1) >> 1) & 1u);
             const int nh = ti.nsplit < ti.rows ? 2 : 1;
             for (int kb = 0; kb < nkb; ++kb) {
@@ -569,8 +609,7 @@ __global__ void __launch_bounds__(GTHREADS, 1) lis_attn_gen_kernel(const __grid_
         if (elect_one()) {
             const uint64_t ones = smem_desc_plain(sa(ONES), 128, 256);
             uint32_t vs = 0, vph = 0, ps = 0, pph = 0;
-            for (int it = 0; it < n; ++it) {
-                const GTile ti = gen_tile(p, t_begin + it, tpb);
+            for (int it = 0; it < n; ++it, ti = gen_next(p, ti)) {
                 const int nh = ti.nsplit < ti.rows ? 2 : 1, par = it & 1;
                 if (it >= 2) mbar_wait(&sh.dfree[par], (uint32_t)((it - 2) >> 1) & 1u, abort_flag);
                 for (int kb = 0; kb < nkb; ++kb) {
@@ -604,8 +643,7 @@ __global__ void __launch_bounds__(GTHREADS, 1) lis_attn_gen_kernel(const __grid_
         // ---------------- copies of the logits tiles
         if (elect_one()) {
             int issued = 0;
-            for (int it = 0; it < n; ++it) {
-                const GTile ti = gen_tile(p, t_begin + it, tpb);
+            for (int it = 0; it < n; ++it, ti = gen_next(p, ti)) {
                 const int lb = p.nlg == 2 ? it & 1 : 0, use = p.nlg == 2 ? it >> 1 : it;
                 const uint32_t bytes = (uint32_t)(ti.rows * p.ld);
                 if (it >= p.nlg) {
@@ -643,7 +681,7 @@ bool gen_layout(const LisArgs &a, GenParams &p, uint32_t &smem)
     const int nb = 2 * a.window - 1;
     if (bias) o = up(o + (uint64_t)nkb * 64 * 8 + (uint64_t)a.heads * nb * nb, 16);
     p.off_r = (uint32_t)o;
-    if (a.region) o += (uint64_t)a.n_windows * Lp;
+    if (a.region) o = up(o + (uint64_t)a.n_windows * (Lp + 1), 16);
     p.off_lg = (uint32_t)o;
     const uint64_t tile = (uint64_t)GM * a.ld_logit;
     p.nlg = o + 2 * tile <= kSmemOptin ? 2 : 1;
