@@ -341,7 +341,7 @@ int attention_path_override()
 }
 
 // The short-row kernel, the long-row kernel that keeps a whole tile's operands, the general one (us at
-// 785 keys, 96 heads, d = 64: general 78, CUDA cores 1129; at 144 keys with bias and mask, 1536 heads: 69
+// 785 keys, 96 heads, d = 64: general 62.5, CUDA cores 1129; at 144 keys with bias and mask, 1536 heads: 56
 // and 440), CUDA cores.  Where two take a shape the first is the faster: it does less per key.
 cudaError_t launch_lis_attention(const LisArgs &la, const AttnVArgs &a, cudaStream_t st)
 {

@@ -32,7 +32,7 @@
 // Algorithm 1), so d is clamped to ne - 1.
 //
 // Issue-bound: about 40 instructions per key.  Swin-S stage 1 with bias and mask (12288
-// heads of 49 keys) 67.8 us -> 58.9: the code from exponents (code_ops), 13 words of keys
+// heads of 49 keys) 67.8 us -> 57.7: the code from exponents (code_ops), 13 words of keys
 // instead of 16, no mask arithmetic in the windows of one region.
 //
 // Every wait is bounded (two seconds), after which the group stops, records a

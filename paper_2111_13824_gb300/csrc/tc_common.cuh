@@ -196,9 +196,10 @@ __device__ __forceinline__ RowSum split_2s(unsigned long long S)
 // 2S = hi + lo (hi rounded toward zero, lo exact) it is RZ(hi + RZ(lo + e)): RZ(lo + e) is the largest
 // multiple of its own last place below lo + e, and the last place of the sum is no finer.  For k = 1
 // (D_1 = 3, not 2) the difference says 1 where the code is 0, for the one key with 3e > 2S that a row can
-// have, its maximum (CodeRow::fix).  6 operations a key where the D_k test takes 10.
+// have, its maximum (CodeRow::fix).  4.5 operations a key where the D_k test takes 10.
 struct CodeRow {
     float hi, lo;
+    uint64_t hi2, lo2, c2;  // {hi, hi}, {lo, lo}, {1.5, 1.5}: made once a row, so that no pair is put together per key
     uint32_t fix;  // 0x0400, to be added to the operand of the maximum when 3 e(0) > 2S, else 0
 };
 
@@ -215,22 +216,29 @@ __device__ __forceinline__ CodeRow code_row(unsigned long long S, float e0)
         r.hi = __int_as_float(((127 + p) << 23) | ((int)(s2 >> sh) & 0x7FFFFF));
         r.lo = __uint2float_rn((uint32_t)s2 & ((1u << sh) - 1u));  // below 2^19
     }
+    asm volatile("mov.b64 %0, {%1, %1};" : "=l"(r.hi2) : "f"(r.hi));
+    asm volatile("mov.b64 %0, {%1, %1};" : "=l"(r.lo2) : "f"(r.lo));
+    asm volatile("mov.b64 %0, 0x3FC000003FC00000;" : "=l"(r.c2));
     r.fix = __fmul_rn(3.0f, e0) > r.hi ? 0x0400u : 0u;  // 3 e0 is representable: 3 e0 > hi says 3 e0 > 2S
     return r;
 }
 
-// a float in [2^(15 - code), 2^(16 - code)) of an i-exp value (before the fix, code not clipped to 15)
-__device__ __forceinline__ float code_pow2(float ef, const CodeRow &r)
-{
-    const float A = __fadd_rz(r.hi, __fadd_rz(r.lo, ef)), g = __fmul_rn(1.5f, ef);
-    return __int_as_float(__float_as_int(g) - __float_as_int(A) + ((143 << 23) - 1));
-}
-
-// the fp16 operands 2^(15 - code) of two keys (low, high half), codes clipped to 15
+// the fp16 operands 2^(15 - code) of two keys (low, high half), codes clipped to 15, the fix not applied:
+// the sums and 3e/2 two at a time (packed fp32: 3 instructions for two keys instead of 6; 8 x 12 heads of 785
+// keys 63.5 -> 62.5 us, Swin-S stage 1 with bias and mask 58.9 -> 57.7), then floats in [2^(15 - code),
+// 2^(16 - code)) from the bits
 __device__ __forceinline__ uint32_t code_ops(float f0, float f1, const CodeRow &r)
 {
+    int a0, a1, g0, g1;
+    asm("{ .reg .b64 f, t, g;\n\t"
+        "mov.b64 f, {%4, %5};\n\tadd.rz.f32x2 t, %6, f;\n\tadd.rz.f32x2 t, %7, t;\n\tmul.rn.f32x2 g, %8, f;\n\t"
+        "mov.b64 {%0, %1}, t;\n\tmov.b64 {%2, %3}, g; }"
+        : "=r"(a0), "=r"(a1), "=r"(g0), "=r"(g1)
+        : "f"(f0), "f"(f1), "l"(r.lo2), "l"(r.hi2), "l"(r.c2));
     uint32_t d;
-    asm("cvt.rz.f16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(code_pow2(f1, r)), "f"(code_pow2(f0, r)));
+    asm("cvt.rz.f16x2.f32 %0, %1, %2;"
+        : "=r"(d)
+        : "f"(__int_as_float(g1 - a1 + ((143 << 23) - 1))), "f"(__int_as_float(g0 - a0 + ((143 << 23) - 1))));
     d &= 0x7C007C00u;
     asm("max.u16x2 %0, %0, %1;" : "+r"(d) : "r"(0x3C003C00u));
     return d;
