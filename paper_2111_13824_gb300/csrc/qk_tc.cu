@@ -19,7 +19,7 @@
 // zeros); per tile, the 128 query rows of Q likewise (A operand).  The keys go
 // through the tensor cores in chunks of 128 (M = 128, N <= 128, K = 64) into four
 // tensor-memory buffers, up to four chunks ahead of the epilogue.  Roles:
-//   warps 0-15 (epilogue): convert the operands, then read each chunk back
+//   warps 0-15 (epilogue): read each chunk back
 //     (warp w: lanes 32 (w % 4) .., columns 32 (w / 4) ..), quantize it and
 //     write the bytes into a staging buffer (or, for strides the tensor store
 //     cannot take, into a shared-memory tile of the output that all of them
@@ -27,9 +27,13 @@
 //   warp 16, one elected lane: the bulk copies of the next tile's Q and head's K
 //     and the MMAs (64 cycles each at N = 128, so it does nothing else);
 //   warp 17, one elected lane: the tensor stores of the staging buffers.
+//   warps 18-21: the operands to fp16, Q one tile ahead (two buffers on the bulk path), K of the
+//     next head chunk by chunk as the MMAs of the current one leave it.
 // They meet only on mbarriers (chunk computed / read, staging written / read,
-// operands converted), so no warp waits at a block barrier for another's MMA
-// issue.  Every wait is bounded: after two seconds the kernel records a timeout
+// operands converted / used), so no warp waits at a block barrier for another's
+// MMA issue, and the epilogue of one tile runs into the next (with the operands
+// converted by the epilogue warps between two tiles, a 512 x 577 x 577 launch, d = 64,
+// took 82 us, now 71; its 175 MB of logits take 47 us to write).  Every wait is bounded: after two seconds the kernel records a timeout
 // status, drains what it issued and returns.
 #include "fqvit_internal.cuh"
 #include "tc_common.cuh"
@@ -53,13 +57,14 @@ constexpr int QKD = 64;          // the MMA's reduction: d padded to 64
 constexpr int QTHREADS = 512;    // epilogue threads (16 warps)
 constexpr int QEPI_WARPS = QTHREADS / 32;
 constexpr int QMMA_WARP = QEPI_WARPS;      // warp 16, lane 0: operand copies and MMAs
-constexpr int QALL = QTHREADS + 64;        // + warp 17, lane 0: tensor stores
-// Register bound of the launch: 18 warps put five on two of the four schedulers, whose register files
-// (16384 each) then allow 96 per thread, the bound a block of 640 threads gets.
-constexpr int QBOUND = 640;
+constexpr int QST_WARP = QMMA_WARP + 1;    // warp 17, lane 0: tensor stores
+constexpr int QCONV_WARP = QST_WARP + 1;   // warps 18-21: operands to fp16
+constexpr int QCONV = 128;                 // converting threads
+constexpr int QALL = 32 * QCONV_WARP + QCONV;
+constexpr int QMAXCH = 5;                  // chunks of the longest row
 constexpr int QMAXL = 640;       // keys of the longest row
 constexpr int QROW = QKD * 2;    // bytes of an fp16 operand row
-constexpr int QNST = 3;          // BULK: staging buffers of a chunk's output (128 x 128 bytes each)
+constexpr int QNST = 4;          // BULK: staging buffers of a chunk's output (128 x 128 bytes each)
 constexpr int QST_BYTES = QM * QNC;
 
 struct QkParams {
@@ -81,7 +86,10 @@ struct QkShared {
     uint64_t sempty[QNBUF];  // every epilogue warp has read buffer b
     uint64_t stfull[QNST];   // every epilogue warp has written staging buffer s (BULK)
     uint64_t stfree[QNST];   // the tensor store of staging buffer s has read it (BULK)
-    uint64_t opsready;       // the tile's Q (and a new head's K) are in the operand layout
+    uint64_t qfull[2];       // a tile's Q is in operand buffer i
+    uint64_t qfree[2];       // the MMAs of operand buffer i are done
+    uint64_t kfull[QMAXCH];  // chunk c of a head's K is in the operand layout
+    uint64_t kfree[QMAXCH];  // the head's last MMAs of chunk c are done
     uint64_t fin, qload, kload;
     uint32_t tmem;
     int abort_flag;
@@ -148,6 +156,34 @@ __device__ __forceinline__ int logit_of(uint32_t acc_bits, const QkParams &p, ui
     }
 }
 
+// eight codes a step of rows [row0, row0 + rows) (those at or past nrows zero) to the swizzled fp16 layout,
+// by the QCONV converting threads (t: 0 ..), eight steps' loads ahead of their conversion
+template <bool SHARED>
+__device__ __forceinline__ void convert_rows(const unsigned char *src, int64_t ld, int row0, int rows, int nrows, int d,
+                                             unsigned char *dst, __half2 z, int t)
+{
+    const int c = t & 7;
+    for (int r = t >> 3; r < rows; r += 8 * (QCONV / 8)) {
+        uint2 w[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int row = row0 + r + u * (QCONV / 8);
+            w[u] = make_uint2(0, 0);
+            if (row < nrows && r + u * (QCONV / 8) < rows && 8 * c < d) {
+                const uint2 *p = reinterpret_cast<const uint2 *>(src + (size_t)row * ld + 8 * c);
+                w[u] = SHARED ? *p : __ldg(p);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int x = r + u * (QCONV / 8), row = row0 + x;
+            if (x >= rows) break;
+            *reinterpret_cast<uint4 *>(dst + x * QROW + ((c ^ (row & 7)) << 4)) =
+                row < nrows && 8 * c < d ? codes_to_h8(w[u], z) : make_uint4(0, 0, 0, 0);
+        }
+    }
+}
+
 // BULK: Q and K rows reach shared memory as int8 by bulk copies one tile (one head) ahead of
 // their conversion (strides of at most 64 bytes, multiples of 16), and each chunk's 128 x 128
 // output bytes leave through one of QNST staging buffers (128-byte swizzle) by a tensor store
@@ -155,15 +191,16 @@ __device__ __forceinline__ int logit_of(uint32_t acc_bits, const QkParams &p, ui
 // one chunk overlaps the work on the next.  Else each thread loads its codes from global
 // memory as it converts them, and the tile's output is copied out from a shared-memory tile.
 template <bool FOLD, bool BULK>
-__global__ void __launch_bounds__(QBOUND, 1)
+__global__ void __launch_bounds__(QALL, 1)
     qk_logits_tc_kernel(const __grid_constant__ QkParams p, const __grid_constant__ CUtensorMap tmap)
 {
     extern __shared__ unsigned char dsm_raw[];
     __shared__ QkShared sh;
     unsigned char *base = dsm_raw + ((1024u - (sa(dsm_raw) & 1023u)) & 1023u);
     unsigned char *KS = base;                            // QMAXL x 128 B (keys, fp16, swizzled)
-    unsigned char *QS = KS + QMAXL * QROW;               // QM x 128 B
-    unsigned char *OS = QS + QM * QROW;                  // BULK: QNST x 16 KB staging; else QM x ld bytes
+    constexpr int NQ = BULK ? 2 : 1;                     // operand buffers of Q
+    unsigned char *QS = KS + QMAXL * QROW;               // NQ x QM x 128 B
+    unsigned char *OS = QS + NQ * QM * QROW;             // BULK: QNST x 16 KB staging; else QM x ld bytes
     unsigned char *KST = OS + (BULK ? (size_t)QNST * QST_BYTES : (size_t)QM * p.ld);  // BULK: L x ld_k int8
     unsigned char *QST = KST + (size_t)QMAXL * 64;       // BULK: QM x ld_q int8 of the next tile
 
@@ -179,7 +216,14 @@ __global__ void __launch_bounds__(QBOUND, 1)
             mbar_init(&sh.stfull[s], QEPI_WARPS);
             mbar_init(&sh.stfree[s], 1);
         }
-        mbar_init(&sh.opsready, QEPI_WARPS);
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&sh.qfull[i], QCONV / 32);
+            mbar_init(&sh.qfree[i], 1);
+        }
+        for (int c = 0; c < QMAXCH; ++c) {
+            mbar_init(&sh.kfull[c], QCONV / 32);
+            mbar_init(&sh.kfree[c], 1);
+        }
         mbar_init(&sh.fin, 1);
         mbar_init(&sh.qload, 1);
         mbar_init(&sh.kload, 1);
@@ -210,59 +254,18 @@ __global__ void __launch_bounds__(QBOUND, 1)
     pdl_wait();  // the set-up above touched no global memory
 
     if (warp < QEPI_WARPS) {
-        // ---------------- epilogue warps: operands in, accumulators out
-        const __half2 zq2 = __half2half2(__int2half_rn(p.zp_q)), zk2 = __half2half2(__int2half_rn(p.zp_k));
+        // ---------------- epilogue warps: accumulators out
         // the requantization's constants in registers (an integer multiply-add takes one constant-bank operand)
         uint32_t rn2 = (uint32_t)p.n2, rc1 = p.c1;
         int rn1 = p.n1;
         asm volatile("" : "+r"(rn2), "+r"(rc1), "+r"(rn1));
         const int qr = 32 * (warp & 3) + lane;  // tile row of this thread
         const int g = warp >> 2;                // 32-column group of a chunk
-        uint32_t qph = 0, kph = 0;              // BULK: phases of the copy barriers waited for
         uint32_t gc = 0;                        // chunks are numbered across the CTA's tiles
-        int cur_bh = -1;
         for (int64_t t = t_begin; t < t_end; ++t) {
             const int bh = (int)(t / tpb);
             const int r0 = (int)(t - (int64_t)bh * tpb) * QM;
-            // ---- operands: K of a new head, the tile's Q rows (8 values = 16 bytes of fp16 per item).
-            //      The MMAs of the previous tile, which read them, have completed: its last chunk was
-            //      waited for below.
             bool bad = false;
-            if (bh != cur_bh) {
-                if (BULK) {
-                    bad = !mbar_wait_warp(&sh.kload, kph & 1, abort_flag);
-                    ++kph;
-                }
-                for (int x = tid; x < L16 * 8 && !bad; x += QTHREADS) {
-                    const int key = x >> 3, c = x & 7;
-                    uint4 h = make_uint4(0, 0, 0, 0);
-                    if (key < L && 8 * c < d) {
-                        const uint2 w = BULK ? *reinterpret_cast<const uint2 *>(KST + key * p.ld_k + 8 * c)
-                                             : __ldg(reinterpret_cast<const uint2 *>(p.k + ((size_t)bh * L + key) * p.ld_k + 8 * c));
-                        h = codes_to_h8(w, zk2);
-                    }
-                    *reinterpret_cast<uint4 *>(KS + key * QROW + ((c ^ (key & 7)) << 4)) = h;
-                }
-                cur_bh = bh;
-            }
-            if (BULK && !bad) {
-                bad = !mbar_wait_warp(&sh.qload, qph & 1, abort_flag);
-                ++qph;
-            }
-            for (int x = tid; x < QM * 8 && !bad; x += QTHREADS) {
-                const int r = x >> 3, c = x & 7;
-                uint4 h = make_uint4(0, 0, 0, 0);
-                if (r0 + r < L && 8 * c < d) {
-                    const uint2 w = BULK ? *reinterpret_cast<const uint2 *>(QST + r * p.ld_q + 8 * c)
-                                         : __ldg(reinterpret_cast<const uint2 *>(p.q + ((size_t)bh * L + r0 + r) * p.ld_q + 8 * c));
-                    h = codes_to_h8(w, zq2);
-                }
-                *reinterpret_cast<uint4 *>(QS + r * QROW + ((c ^ (r & 7)) << 4)) = h;
-            }
-            fence_async_smem();  // the operands are read by the MMAs (and the staging areas refilled)
-            tc_fence_before();
-            __syncwarp();
-            if (!bad && lane == 0) mbar_arrive(&sh.opsready);
             // ---- chunks: read back, quantize, into the output staging (or tile)
             for (int c = 0; c < nch && !bad; ++c, ++gc) {
                 const uint32_t b = gc % QNBUF, s = gc % QNST;
@@ -330,9 +333,8 @@ __global__ void __launch_bounds__(QBOUND, 1)
             }
             // ---- (without BULK) the tile's rows to global memory (contiguous there): 16 bytes per
             //      thread and step, each warp's stores one contiguous 512-byte run.  Every epilogue
-            //      thread reaches this barrier, which also tells each of them whether any gave up; the
-            //      next tile's chunks are computed only after every epilogue warp has arrived on
-            //      opsready again, so after these copies.
+            //      thread reaches the first barrier, which also tells each of them whether any gave up;
+            //      after the second the next tile's rows may be written.
             if (!BULK) {
                 uint32_t any_bad;
                 asm volatile(
@@ -345,6 +347,7 @@ __global__ void __launch_bounds__(QBOUND, 1)
                 int8_t *gdst = p.out + ((size_t)bh * L + r0) * p.ld;
                 for (int64_t x = 16 * (int64_t)tid; x < bytes; x += 16 * QTHREADS)
                     *reinterpret_cast<uint4 *>(gdst + x) = *reinterpret_cast<const uint4 *>(OS + x);
+                asm volatile("bar.sync 1, %0;" ::"n"(QTHREADS) : "memory");
             } else if (bad) {
                 break;
             }
@@ -367,9 +370,9 @@ __global__ void __launch_bounds__(QBOUND, 1)
                 mbar_expect_tx(&sh.kload, bytes);
                 bulk_g2s(KST, p.k + (size_t)bk * L * p.ld_k, bytes, &sh.kload);
             };
-            // a copy is issued only once the operands it replaces were converted (opsready), so at
-            // most one is in flight on each barrier
-            uint32_t qiss = 0, kiss = 0, issued = 0, gc = 0;
+            // a copy is issued only once the operands it replaces were converted (qfull, the last kfull),
+            // so at most one is in flight on each barrier
+            uint32_t qiss = 0, kiss = 0, issued = 0, gc = 0, nh = 0;  // nh: heads before this one
             if (BULK && t_begin < t_end) {
                 copy_q(t_begin);
                 copy_k((int)(t_begin / tpb));
@@ -377,16 +380,16 @@ __global__ void __launch_bounds__(QBOUND, 1)
             }
             bool ok = true;
             for (int64_t t = t_begin; t < t_end && ok; ++t) {
-                ok = mbar_wait(&sh.opsready, (uint32_t)(t - t_begin) & 1, abort_flag);
+                const uint32_t i = (uint32_t)(t - t_begin), qb = i % NQ;
+                const int head = (int)(t / tpb);
+                const bool first = t == t_begin || (int)((t - 1) / tpb) != head;
+                const bool last = t + 1 == t_end || (int)((t + 1) / tpb) != head;
+                if (first && t != t_begin) ++nh;
+                ok = mbar_wait(&sh.qfull[qb], (i / NQ) & 1, abort_flag);
                 if (!ok) break;
-                tc_fence_after();
-                if (BULK && t + 1 < t_end) {  // the staging areas were converted: the next tile's operands
+                if (BULK && t + 1 < t_end) {  // the staging area was converted: the next tile's Q
                     copy_q(t + 1);
                     ++qiss;
-                    if ((int)((t + 1) / tpb) != (int)(t / tpb)) {
-                        copy_k((int)((t + 1) / tpb));
-                        ++kiss;
-                    }
                 }
                 for (int c = 0; c < nch; ++c, ++gc) {
                     const uint32_t b = gc % QNBUF;
@@ -395,16 +398,26 @@ __global__ void __launch_bounds__(QBOUND, 1)
                         ok = false;
                         break;
                     }
+                    if (first && !mbar_wait(&sh.kfull[c], nh & 1, abort_flag)) {
+                        ok = false;
+                        break;
+                    }
+                    if (BULK && first && c + 1 == nch && ((int64_t)head + 1) * tpb < t_end) {
+                        copy_k(head + 1);  // the staging area was converted: the next head's K
+                        ++kiss;
+                    }
                     tc_fence_after();
                     const int n = min(QNC, L16 - c * QNC);
-                    const uint32_t a0 = sa(QS), b0 = sa(KS) + (uint32_t)(c * QNC * QROW);
+                    const uint32_t a0 = sa(QS) + qb * (QM * QROW), b0 = sa(KS) + (uint32_t)(c * QNC * QROW);
 #pragma unroll
                     for (int s = 0; s < QKD / 16; ++s)
                         mma_f16_ss(tmem + b * QNC, smem_desc(a0 + 32 * s, 16, 1024), smem_desc(b0 + 32 * s, 16, 1024),
                                    idesc(n), s != 0);
                     mma_commit(&sh.sfull[b]);
+                    if (last) mma_commit(&sh.kfree[c]);
                     ++issued;
                 }
+                mma_commit(&sh.qfree[qb]);
             }
             // every copy and every MMA issued has completed before shared and tensor memory are released
             if (BULK && qiss > 0) mbar_wait(&sh.qload, (qiss - 1) & 1, abort_flag, false);
@@ -414,28 +427,65 @@ __global__ void __launch_bounds__(QBOUND, 1)
                 mbar_wait(&sh.fin, 0, abort_flag, false);
             }
         }
-    } else if (BULK && elect_one()) {
-        // ---------------- warp 17, lane 0: the tensor stores of the chunks' staging buffers
-        uint32_t gc = 0;
+    } else if (warp == QST_WARP) {
+        // ---------------- warp 17, one lane: the tensor stores of the chunks' staging buffers, one in
+        // flight while the next is issued
+        if (BULK && elect_one()) {
+            uint32_t gc = 0;
+            bool ok = true;
+            for (int64_t t = t_begin; t < t_end && ok; ++t) {
+                const int bh = (int)(t / tpb);
+                const int r0 = (int)(t - (int64_t)bh * tpb) * QM;
+                for (int c = 0; c < nch; ++c, ++gc) {
+                    const uint32_t s = gc % QNST;
+                    ok = mbar_wait(&sh.stfull[s], (gc / QNST) & 1, abort_flag);
+                    if (!ok) break;
+                    // chunk c of the tile: columns c 128 .., rows r0 .., head bh
+                    asm volatile(
+                        "cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(&tmap),
+                        "r"(c * QNC), "r"(r0), "r"(bh), "r"(sa(OS + (size_t)s * QST_BYTES))
+                        : "memory");
+                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                    asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");  // the one before has been read
+                    if (gc > 0) mbar_arrive(&sh.stfree[(gc - 1) % QNST]);
+                }
+            }
+            asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");  // every store has completed
+        }
+    } else {
+        // ---------------- warps 18-21: K of a new head, chunk by chunk as the last head's MMAs leave it, and
+        // the tile's Q, one tile ahead of the MMAs
+        const __half2 zq2 = __half2half2(__int2half_rn(p.zp_q)), zk2 = __half2half2(__int2half_rn(p.zp_k));
+        const int ct = tid - 32 * QCONV_WARP;
+        uint32_t nh = 0;
+        auto done = [&](uint64_t *b) {
+            fence_async_smem();  // the operands are read by the MMAs, the staging areas refilled by copies
+            __syncwarp();
+            if (lane == 0) mbar_arrive(b);
+        };
         bool ok = true;
         for (int64_t t = t_begin; t < t_end && ok; ++t) {
+            const uint32_t i = (uint32_t)(t - t_begin), qb = i % NQ;
             const int bh = (int)(t / tpb);
             const int r0 = (int)(t - (int64_t)bh * tpb) * QM;
-            for (int c = 0; c < nch; ++c, ++gc) {
-                const uint32_t s = gc % QNST;
-                ok = mbar_wait(&sh.stfull[s], (gc / QNST) & 1, abort_flag);
-                if (!ok) break;
-                // chunk c of the tile: columns c 128 .., rows r0 .., head bh
-                asm volatile(
-                    "cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(&tmap),
-                    "r"(c * QNC), "r"(r0), "r"(bh), "r"(sa(OS + (size_t)s * QST_BYTES))
-                    : "memory");
-                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-                asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // the buffer has been read
-                mbar_arrive(&sh.stfree[s]);
+            if (i >= NQ) ok = mbar_wait_warp(&sh.qfree[qb], (i / NQ - 1) & 1, abort_flag);
+            if (BULK && ok) ok = mbar_wait_warp(&sh.qload, i & 1, abort_flag);
+            if (!ok) break;
+            convert_rows<BULK>(BULK ? QST - (size_t)r0 * p.ld_q : (const unsigned char *)p.q + (size_t)bh * L * p.ld_q,
+                               p.ld_q, r0, QM, L, d, QS + qb * (QM * QROW), zq2, ct);
+            done(&sh.qfull[qb]);
+            if (i == 0 || r0 == 0) {
+                if (BULK) ok = mbar_wait_warp(&sh.kload, nh & 1, abort_flag);
+                for (int c = 0; c < nch && ok; ++c) {
+                    if (nh > 0) ok = mbar_wait_warp(&sh.kfree[c], (nh - 1) & 1, abort_flag);
+                    if (!ok) break;
+                    convert_rows<BULK>(BULK ? KST : (const unsigned char *)p.k + (size_t)bh * L * p.ld_k, p.ld_k, c * QNC,
+                                       min(QNC, L16 - c * QNC), L, d, KS + c * QNC * QROW, zk2, ct);
+                    done(&sh.kfull[c]);
+                }
+                ++nh;
             }
         }
-        asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");  // every store has completed
     }
     tc_fence_before();
     __syncthreads();
@@ -446,7 +496,7 @@ __global__ void __launch_bounds__(QBOUND, 1)
 
 size_t qk_smem_bytes(int64_t ld, bool bulk)
 {
-    return 1024 + (size_t)QMAXL * QROW + (size_t)QM * QROW +
+    return 1024 + (size_t)QMAXL * QROW + (size_t)(bulk ? 2 : 1) * QM * QROW +
            (bulk ? (size_t)QNST * QST_BYTES + (size_t)QMAXL * 64 + QM * 64 : (size_t)QM * ld);
 }
 
