@@ -19,21 +19,27 @@
 // zeros); per tile, the 128 query rows of Q likewise (A operand).  The keys go
 // through the tensor cores in chunks of 128 (M = 128, N <= 128, K = 64) into four
 // tensor-memory buffers, up to four chunks ahead of the epilogue.  Roles:
-//   warps 0-15 (epilogue): read each chunk back
-//     (warp w: lanes 32 (w % 4) .., columns 32 (w / 4) ..), quantize it and
+//   warps 0-15 (epilogue), two groups of eight taking every other chunk: read it
+//     back (warp w: lanes 32 (w % 4) .., columns 64 (w / 4 % 2) ..), quantize it and
 //     write the bytes into a staging buffer (or, for strides the tensor store
 //     cannot take, into a shared-memory tile of the output that all of them
-//     copy out with coalesced 16-byte stores);
+//     copy out with coalesced 16-byte stores).  One group waits for its
+//     accumulators while the other computes;
 //   warp 16, one elected lane: the bulk copies of the next tile's Q and head's K
 //     and the MMAs (64 cycles each at N = 128, so it does nothing else);
-//   warp 17, one elected lane: the tensor stores of the staging buffers.
-//   warps 18-21: the operands to fp16, Q one tile ahead (two buffers on the bulk path), K of the
-//     next head chunk by chunk as the MMAs of the current one leave it.
+//   warp 17, one elected lane: the tensor stores of the staging buffers;
+//   warps 18-25: the operands to fp16, Q one tile ahead (two buffers on the bulk
+//     path), K of the next head chunk by chunk as the MMAs of the current one
+//     leave it.
 // They meet only on mbarriers (chunk computed / read, staging written / read,
 // operands converted / used), so no warp waits at a block barrier for another's
-// MMA issue, and the epilogue of one tile runs into the next (with the operands
-// converted by the epilogue warps between two tiles, a 512 x 577 x 577 launch, d = 64,
-// took 82 us, now 71; its 175 MB of logits take 47 us to write).  Every wait is bounded: after two seconds the kernel records a timeout
+// MMA issue, and the epilogue of one tile runs into the next.
+//
+// Measured, 512 x 577 x 577, d = 64 (175 MB of logits, 47 us to write): 82 us with the
+// operands converted by the epilogue warps between two tiles, 71 with four converting
+// warps of their own, 59 with eight, 16-byte steps and one subtraction a pair of codes.
+// Without the conversion (timed alone) 54, without the stores 4 less, the MMAs hidden.
+// Every wait is bounded: after two seconds the kernel records a timeout
 // status, drains what it issued and returns.
 #include "fqvit_internal.cuh"
 #include "tc_common.cuh"
@@ -58,8 +64,8 @@ constexpr int QTHREADS = 512;    // epilogue threads (16 warps)
 constexpr int QEPI_WARPS = QTHREADS / 32;
 constexpr int QMMA_WARP = QEPI_WARPS;      // warp 16, lane 0: operand copies and MMAs
 constexpr int QST_WARP = QMMA_WARP + 1;    // warp 17, lane 0: tensor stores
-constexpr int QCONV_WARP = QST_WARP + 1;   // warps 18-21: operands to fp16
-constexpr int QCONV = 128;                 // converting threads
+constexpr int QCONV_WARP = QST_WARP + 1;   // warps 18-25: operands to fp16
+constexpr int QCONV = 256;                 // converting threads
 constexpr int QALL = 32 * QCONV_WARP + QCONV;
 constexpr int QMAXCH = 5;                  // chunks of the longest row
 constexpr int QMAXL = 640;       // keys of the longest row
@@ -102,14 +108,16 @@ __device__ __forceinline__ uint32_t pack_sat_s8(int hi, int lo, uint32_t c)
     return d;
 }
 
-// eight int8 codes minus a zero point -> eight fp16 values (exact: -255 .. 255)
-__device__ __forceinline__ uint4 codes_to_h8(uint2 w, __half2 z)
+// eight int8 codes minus a zero point -> eight fp16 values (exact: -255 .. 255).  A biased byte under the
+// high byte 0x64 is 1024 + (code + 128); z is 1152 + the zero point, exact too.
+__device__ __forceinline__ uint4 codes_to_h8(uint32_t w0, uint32_t w1, __half2 z)
 {
-    const uint32_t x0 = w.x ^ 0x80808080u, x1 = w.y ^ 0x80808080u;
-    uint32_t h[4] = {i8x2_to_h2(x0, 0x5140), i8x2_to_h2(x0, 0x7362), i8x2_to_h2(x1, 0x5140), i8x2_to_h2(x1, 0x7362)};
+    const uint32_t x0 = w0 ^ 0x80808080u, x1 = w1 ^ 0x80808080u;
+    uint32_t h[4] = {__byte_perm(x0, 0x64646464u, 0x5140), __byte_perm(x0, 0x64646464u, 0x7362),
+                     __byte_perm(x1, 0x64646464u, 0x5140), __byte_perm(x1, 0x64646464u, 0x7362)};
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        __half2 t = __hsub2(*reinterpret_cast<const __half2 *>(&h[i]), z);
+        const __half2 t = __hsub2(*reinterpret_cast<const __half2 *>(&h[i]), z);
         h[i] = *reinterpret_cast<const uint32_t *>(&t);
     }
     return make_uint4(h[0], h[1], h[2], h[3]);
@@ -156,31 +164,42 @@ __device__ __forceinline__ int logit_of(uint32_t acc_bits, const QkParams &p, ui
     }
 }
 
-// eight codes a step of rows [row0, row0 + rows) (those at or past nrows zero) to the swizzled fp16 layout,
-// by the QCONV converting threads (t: 0 ..), eight steps' loads ahead of their conversion
+// Rows [row0, row0 + rows) (rows <= 128; those at or past nrows zero) to the swizzled fp16 layout by the QCONV
+// converting threads (t: 0 ..), 16 codes a step, every step's load ahead of the conversions.  SHARED: 16-byte
+// rows in shared memory.
 template <bool SHARED>
 __device__ __forceinline__ void convert_rows(const unsigned char *src, int64_t ld, int row0, int rows, int nrows, int d,
                                              unsigned char *dst, __half2 z, int t)
 {
-    const int c = t & 7;
-    for (int r = t >> 3; r < rows; r += 8 * (QCONV / 8)) {
-        uint2 w[8];
+    constexpr int STEP = QCONV / 4, U = QNC / STEP;
+    const int c = t & 3;  // codes 16 c .. 16 c + 15 of a row
+    const uint4 zero = make_uint4(0, 0, 0, 0);
+    uint4 w[U];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int row = row0 + r + u * (QCONV / 8);
-            w[u] = make_uint2(0, 0);
-            if (row < nrows && r + u * (QCONV / 8) < rows && 8 * c < d) {
-                const uint2 *p = reinterpret_cast<const uint2 *>(src + (size_t)row * ld + 8 * c);
-                w[u] = SHARED ? *p : __ldg(p);
+    for (int u = 0; u < U; ++u) {
+        const int x = (t >> 2) + u * STEP, row = row0 + x;
+        w[u] = zero;
+        if (x < rows && row < nrows && 16 * c < d) {
+            const unsigned char *p = src + (size_t)row * ld + 16 * c;
+            if (SHARED) {
+                w[u] = *reinterpret_cast<const uint4 *>(p);
+            } else {
+                const uint2 a = __ldg(reinterpret_cast<const uint2 *>(p));
+                const uint2 b = 16 * c + 8 < d ? __ldg(reinterpret_cast<const uint2 *>(p) + 1) : make_uint2(0, 0);
+                w[u] = make_uint4(a.x, a.y, b.x, b.y);
             }
         }
+    }
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int x = r + u * (QCONV / 8), row = row0 + x;
-            if (x >= rows) break;
-            *reinterpret_cast<uint4 *>(dst + x * QROW + ((c ^ (row & 7)) << 4)) =
-                row < nrows && 8 * c < d ? codes_to_h8(w[u], z) : make_uint4(0, 0, 0, 0);
-        }
+    for (int u = 0; u < U; ++u) {
+        const int x = (t >> 2) + u * STEP, row = row0 + x;
+        if (x >= rows) break;
+        const bool in = row < nrows;
+        unsigned char *o = dst + x * QROW;
+        *reinterpret_cast<uint4 *>(o + (((2 * c) ^ (row & 7)) << 4)) =
+            in && 16 * c < d ? codes_to_h8(w[u].x, w[u].y, z) : zero;
+        *reinterpret_cast<uint4 *>(o + (((2 * c + 1) ^ (row & 7)) << 4)) =
+            in && 16 * c + 8 < d ? codes_to_h8(w[u].z, w[u].w, z) : zero;
     }
 }
 
@@ -210,10 +229,10 @@ __global__ void __launch_bounds__(QALL, 1)
     if (tid == 0) {
         for (int b = 0; b < QNBUF; ++b) {
             mbar_init(&sh.sfull[b], 1);
-            mbar_init(&sh.sempty[b], QEPI_WARPS);
+            mbar_init(&sh.sempty[b], QEPI_WARPS / 2);
         }
         for (int s = 0; s < QNST; ++s) {
-            mbar_init(&sh.stfull[s], QEPI_WARPS);
+            mbar_init(&sh.stfull[s], QEPI_WARPS / 2);
             mbar_init(&sh.stfree[s], 1);
         }
         for (int i = 0; i < 2; ++i) {
@@ -260,7 +279,8 @@ __global__ void __launch_bounds__(QALL, 1)
         int rn1 = p.n1;
         asm volatile("" : "+r"(rn2), "+r"(rc1), "+r"(rn1));
         const int qr = 32 * (warp & 3) + lane;  // tile row of this thread
-        const int g = warp >> 2;                // 32-column group of a chunk
+        const int g = (warp >> 2) & 1;          // 64-column half of a chunk
+        const int half = warp >> 3;             // which chunks: every other one, the other way round in the next tile
         uint32_t gc = 0;                        // chunks are numbered across the CTA's tiles
         for (int64_t t = t_begin; t < t_end; ++t) {
             const int bh = (int)(t / tpb);
@@ -268,6 +288,7 @@ __global__ void __launch_bounds__(QALL, 1)
             bool bad = false;
             // ---- chunks: read back, quantize, into the output staging (or tile)
             for (int c = 0; c < nch && !bad; ++c, ++gc) {
+                if (((c ^ (int)(t - t_begin)) & 1) != half) continue;
                 const uint32_t b = gc % QNBUF, s = gc % QNST;
                 bad = !mbar_wait_warp(&sh.sfull[b], (gc / QNBUF) & 1, abort_flag);
                 // BULK: the store of chunk gc - QNST has read this staging buffer
@@ -275,52 +296,55 @@ __global__ void __launch_bounds__(QALL, 1)
                     bad = !mbar_wait_warp(&sh.stfree[s], ((gc - QNST) / QNST) & 1, abort_flag);
                 if (bad) break;
                 tc_fence_after();
-                const int col0 = c * QNC + 32 * g;  // first key of this warp's 32 columns
                 // BULK: this chunk's staging buffer, 16-byte unit u of tile row qr at u ^ (qr % 8)
                 unsigned char *srow = OS + (size_t)s * QST_BYTES + qr * QNC;
-                if (BULK && col0 >= L16 && col0 < p.ld) {  // bytes past the keys, inside the row
-                    *reinterpret_cast<uint4 *>(srow + (((2 * g) ^ (qr & 7)) << 4)) = make_uint4(0, 0, 0, 0);
-                    *reinterpret_cast<uint4 *>(srow + (((2 * g + 1) ^ (qr & 7)) << 4)) = make_uint4(0, 0, 0, 0);
-                }
-                if (col0 < L16) {
-                    uint32_t v[32];
-                    tmem_ld32(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(b * QNC + 32 * g), v);
-                    tmem_wait_ld();
-                    uint32_t w[8];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        int l0, l1, l2, l3;
-                        if (FOLD) {  // the magic additions two at a time
-                            uint32_t x0, x1, x2, x3;
-                            add_magic2(v[4 * i], v[4 * i + 1], x0, x1);
-                            add_magic2(v[4 * i + 2], v[4 * i + 3], x2, x3);
-                            l0 = logit_of_biased(x0, rn2, rc1, rn1);
-                            l1 = logit_of_biased(x1, rn2, rc1, rn1);
-                            l2 = logit_of_biased(x2, rn2, rc1, rn1);
-                            l3 = logit_of_biased(x3, rn2, rc1, rn1);
-                        } else {
-                            l0 = logit_of<FOLD>(v[4 * i], p, rn2, rc1, rn1);
-                            l1 = logit_of<FOLD>(v[4 * i + 1], p, rn2, rc1, rn1);
-                            l2 = logit_of<FOLD>(v[4 * i + 2], p, rn2, rc1, rn1);
-                            l3 = logit_of<FOLD>(v[4 * i + 3], p, rn2, rc1, rn1);
-                        }
-                        w[i] = pack_sat_s8(l1, l0, pack_sat_s8(l3, l2, 0u));
+#pragma unroll 1
+                for (int hc = 0; hc < 2; ++hc) {
+                    const int u = 4 * g + 2 * hc, col0 = c * QNC + 16 * u;  // 32 columns: first unit, first key
+                    if (BULK && col0 >= L16 && col0 < p.ld) {  // bytes past the keys, inside the row
+                        *reinterpret_cast<uint4 *>(srow + ((u ^ (qr & 7)) << 4)) = make_uint4(0, 0, 0, 0);
+                        *reinterpret_cast<uint4 *>(srow + (((u + 1) ^ (qr & 7)) << 4)) = make_uint4(0, 0, 0, 0);
                     }
-                    if (col0 + 32 > L) {  // keys at or past L: zero bytes (the last chunk only)
+                    if (col0 < L16) {
+                        uint32_t v[32];
+                        tmem_ld32(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(b * QNC + 64 * g + 32 * hc), v);
+                        tmem_wait_ld();
+                        uint32_t w[8];
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
-                            const int k0 = col0 + 4 * i;
-                            if (k0 + 4 > L) w[i] &= k0 >= L ? 0u : (0xFFFFFFFFu >> (32 - 8 * (L - k0)));
+                            int l0, l1, l2, l3;
+                            if (FOLD) {  // the magic additions two at a time
+                                uint32_t x0, x1, x2, x3;
+                                add_magic2(v[4 * i], v[4 * i + 1], x0, x1);
+                                add_magic2(v[4 * i + 2], v[4 * i + 3], x2, x3);
+                                l0 = logit_of_biased(x0, rn2, rc1, rn1);
+                                l1 = logit_of_biased(x1, rn2, rc1, rn1);
+                                l2 = logit_of_biased(x2, rn2, rc1, rn1);
+                                l3 = logit_of_biased(x3, rn2, rc1, rn1);
+                            } else {
+                                l0 = logit_of<FOLD>(v[4 * i], p, rn2, rc1, rn1);
+                                l1 = logit_of<FOLD>(v[4 * i + 1], p, rn2, rc1, rn1);
+                                l2 = logit_of<FOLD>(v[4 * i + 2], p, rn2, rc1, rn1);
+                                l3 = logit_of<FOLD>(v[4 * i + 3], p, rn2, rc1, rn1);
+                            }
+                            w[i] = pack_sat_s8(l1, l0, pack_sat_s8(l3, l2, 0u));
                         }
-                    }
-                    if (BULK) {  // units past L16 hold zeros (w is masked past L) or lie past ld (clipped)
-                        *reinterpret_cast<uint4 *>(srow + (((2 * g) ^ (qr & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
-                        *reinterpret_cast<uint4 *>(srow + (((2 * g + 1) ^ (qr & 7)) << 4)) =
-                            col0 + 16 < L16 ? make_uint4(w[4], w[5], w[6], w[7]) : make_uint4(0, 0, 0, 0);
-                    } else {
-                        unsigned char *dst = OS + (size_t)qr * p.ld + col0;
-                        *reinterpret_cast<uint4 *>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
-                        if (col0 + 16 < L16) *reinterpret_cast<uint4 *>(dst + 16) = make_uint4(w[4], w[5], w[6], w[7]);
+                        if (col0 + 32 > L) {  // keys at or past L: zero bytes (the last chunk only)
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) {
+                                const int k0 = col0 + 4 * i;
+                                if (k0 + 4 > L) w[i] &= k0 >= L ? 0u : (0xFFFFFFFFu >> (32 - 8 * (L - k0)));
+                            }
+                        }
+                        if (BULK) {  // units past L16 hold zeros (w is masked past L) or lie past ld (clipped)
+                            *reinterpret_cast<uint4 *>(srow + ((u ^ (qr & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+                            *reinterpret_cast<uint4 *>(srow + (((u + 1) ^ (qr & 7)) << 4)) =
+                                col0 + 16 < L16 ? make_uint4(w[4], w[5], w[6], w[7]) : make_uint4(0, 0, 0, 0);
+                        } else {
+                            unsigned char *dst = OS + (size_t)qr * p.ld + col0;
+                            *reinterpret_cast<uint4 *>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+                            if (col0 + 16 < L16) *reinterpret_cast<uint4 *>(dst + 16) = make_uint4(w[4], w[5], w[6], w[7]);
+                        }
                     }
                 }
                 if (BULK) fence_async_smem();  // the staging bytes are read by the tensor store
@@ -453,9 +477,9 @@ __global__ void __launch_bounds__(QALL, 1)
             asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");  // every store has completed
         }
     } else {
-        // ---------------- warps 18-21: K of a new head, chunk by chunk as the last head's MMAs leave it, and
+        // ---------------- warps 18-25: K of a new head, chunk by chunk as the last head's MMAs leave it, and
         // the tile's Q, one tile ahead of the MMAs
-        const __half2 zq2 = __half2half2(__int2half_rn(p.zp_q)), zk2 = __half2half2(__int2half_rn(p.zp_k));
+        const __half2 zq2 = __half2half2(__int2half_rn(1152 + p.zp_q)), zk2 = __half2half2(__int2half_rn(1152 + p.zp_k));
         const int ct = tid - 32 * QCONV_WARP;
         uint32_t nh = 0;
         auto done = [&](uint64_t *b) {
