@@ -30,7 +30,9 @@
 //     bytes from the replicated maximum), the i-exp row sum from a table
 //     indexed by d, the row's 15 code thresholds, the row's operand table (the
 //     fp16 operand 2^(15 - code) of every d), and the operands of the row's
-//     keys, looked up by d, straight into tensor memory.
+//     keys, looked up by d, straight into tensor memory.  Rows of up to 384 keys (DIRECT) have no thresholds and
+//     no operand table: each key's operand comes from its i-exp value (code_ops, tc_common.cuh), the table's
+//     operand half holds 32 copies of the fp32 values, and only the four warps of 32 rows ever meet.
 //   warps 16-19, one per tensor-memory lane quarter: the accumulators of the
 //     previous tile out of tensor memory into global memory, V of a new head
 //     into the fp16 B operand in shared memory, the tile's MMAs (warp 16, lane
@@ -86,6 +88,12 @@ constexpr int TCOPY_WARP = TEPI_WARP + 1;  //   warp 17 lane 0 also copies the l
 constexpr int TTHREADS = TSOFT + 128;
 constexpr int TMAXKB = 10;                 // key blocks of the longest row
 constexpr int kPackMaxBlocks = 6;          // PACK for 128 <= L <= 384
+// Rows of up to this many 64-key blocks take each key's operand from its i-exp value (code_ops), longer ones
+// from a table per row.  The table costs a thread about 450 instructions and two barriers of all 16 warps a
+// tile, the evaluation about 4 instructions a key.  us per call, table / evaluation (int32 output): 384 heads of
+// 65 keys 14.8 / 11.1, of 128 18.4 / 14.4, of 197 22.9 / 20.4, of 320 42.5 / 38.7; 384 heads of 400 61.4 / 59.8
+// but with 8 bits and a zero point of V 58.9 / 61.0; 512 heads of 577 110.9 / 119.6.
+constexpr int kDirectBlocks = 6;
 
 // Shared memory.  The kernel has no static shared memory, so its dynamic shared memory starts at
 // the first address after the 1 KB the driver reserves (1024; the kernel checks it).  The combined
@@ -235,7 +243,7 @@ struct TcShared {
     int bk0, bkmax;  // bucket number of table entry 0, and of the last entry
     int abort_flag;
     int rising;   // some i-exp value exceeds the one before it (floored constants)
-    int stop;     // set (never cleared) by a softmax thread whose wait gave up
+    int stop[4];  // set (never cleared) by a softmax thread whose wait gave up, for the threads that meet it
     int ew_stop;  // the same for the read-out warps
 };
 
@@ -246,6 +254,13 @@ __device__ __forceinline__ void soft_bar()
 {
     __syncwarp();
     asm volatile("bar.sync 1, %0;" ::"n"(TSOFT) : "memory");
+}
+
+// Named barriers 3 .. 6: the 128 softmax threads of rows 32 k4 .. 32 k4 + 31
+__device__ __forceinline__ void group_bar(int k4)
+{
+    __syncwarp();
+    asm volatile("bar.sync %0, 128;" ::"r"(3 + k4) : "memory");
 }
 
 // Named barrier 2 over the 128 read-out threads
@@ -394,6 +409,7 @@ __device__ __forceinline__ void read_out_row(const TcParams &p, uint32_t etl, ui
 template <int NKB, bool SMALL_E, bool PACK>
 __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
 {
+    constexpr bool DIRECT = NKB <= kDirectBlocks;
     extern __shared__ __align__(1024) unsigned char dsm[];
     TcShared &sh = *reinterpret_cast<TcShared *>(dsm + C_SH);
     uint32_t *ONES = reinterpret_cast<uint32_t *>(dsm + C_ONES);
@@ -408,7 +424,6 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     volatile int *abort_flag = &sh.abort_flag;
-    volatile int *stop_flag = &sh.stop;
     const int L = p.L;
     const int nsteps = (L + 15) >> 4;  // MMA K steps of 16 keys
     pdl_release();
@@ -430,7 +445,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
         mbar_init(&sh.fin, 1);
         sh.abort_flag = 0;
         sh.rising = 0;
-        sh.stop = 0;
+        for (int k = 0; k < 4; ++k) sh.stop[k] = 0;
         sh.ew_stop = 0;
         sh.c = p.ic;
     }
@@ -454,6 +469,9 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
         __syncthreads();
         for (int i = tid; i < 256 * 32; i += blockDim.x)
             sts_u32(kTabAbs + (uint32_t)(i >> 5) * 256u + LUT_BYTE + 4u * (i & 31), e_tmp[i >> 5]);
+        if (DIRECT)
+            for (int i = tid; i < 256 * 32; i += blockDim.x)
+                sts_u32(kTabAbs + (uint32_t)(i >> 5) * 256u + 4u * (i & 31), __float_as_uint(LUTF[i >> 5]));
         for (int d = tid; d < 255; d += blockDim.x)
             if (e_tmp[d] < e_tmp[d + 1]) sh.rising = 1;
     }
@@ -463,7 +481,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
         sh.bk0 = bkmax - (BK_N - 1);
     }
     __syncthreads();  // the copies of the i-exp values read, rising, the bucket range
-    if (!sh.rising) {
+    if (!DIRECT && !sh.rising) {
         // #{d : e(d) > x} by binary search (the values never rise with d)
         auto count_above = [&](float x) -> int {
             int lo = 0;
@@ -500,7 +518,15 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
         const int r = 32 * k4 + lane;                    // row of the tile = tensor-memory lane
         // offset registers of the table lookups (1 << 16 selects the table's 64 K page): this row's byte
         // in a line, and this lane's i-exp copy in a line
-        const uint32_t rowb = 0x10000u | (4u * (uint32_t)lane + (uint32_t)k4);
+        const uint32_t rowb = 0x10000u | (4u * (uint32_t)lane + (DIRECT ? 0u : (uint32_t)k4));
+        volatile int *stop_flag = &sh.stop[DIRECT ? k4 : 0];
+        auto meet = [&]() {  // DIRECT: the threads of these 32 rows; else all, whose rows share the table's words
+            if (DIRECT)
+                group_bar(k4);
+            else
+                soft_bar();
+        };
+        const float e0f = LUTF[0];
         const uint32_t lutb = 0x10000u | (LUT_BYTE + 4u * (uint32_t)lane);
         const uint32_t tlane = tmem + ((uint32_t)(k4 * 32) << 16);
         const bool monotone = !sh.rising;  // codes never fall as d grows
@@ -570,18 +596,20 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
             int m = max(max(sbyte<1>(mo), sbyte<3>(mo)), max((int)(me & 0xFFFFu), (int)(me >> 16)) - 128);
             red_max[q * TM + r] = m;
             if (lbad || wait_bad) *stop_flag = 1;
-            soft_bar();  // A
+            meet();  // A
             if (*stop_flag) break;  // every softmax thread leaves here together
             m = max(max(red_max[r], red_max[TM + r]), max(red_max[2 * TM + r], red_max[3 * TM + r]));
-            // the previous tile's operand table is dead (every thread has passed its lookups): clear
-            // its bytes and the group totals for this tile's thresholds
+            if constexpr (!DIRECT) {
+                // the previous tile's operand table is dead (every thread has passed its lookups): clear
+                // its bytes and the group totals for this tile's thresholds
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const uint32_t c = (uint32_t)(tid + TSOFT * i);
-                sts_zero16(kTabAbs + (c >> 3) * 256u + (c & 7u) * 16u);
+                for (int i = 0; i < 4; ++i) {
+                    const uint32_t c = (uint32_t)(tid + TSOFT * i);
+                    sts_zero16(kTabAbs + (c >> 3) * 256u + (c & 7u) * 16u);
+                }
+                GT[tid] = 0u;
+                if (tid < 32 * GT_LD - TSOFT) GT[TSOFT + tid] = 0u;
             }
-            GT[tid] = 0u;
-            if (tid < 32 * GT_LD - TSOFT) GT[TSOFT + tid] = 0u;
             // ---- distances: byte d = m - q = (m + 128) - (q + 128), four per word, no borrows
             {
                 const uint32_t mrep = (uint32_t)(m + 128) * 0x01010101u;
@@ -636,107 +664,112 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
                 S -= (unsigned long long)npad * lds_u32(((uint32_t)(m + 128) << 8) + lutb);
             }
             red_sum[q * TM + r] = S;
-            soft_bar();  // B
+            meet();  // B
             S = red_sum[r] + red_sum[TM + r] + red_sum[2 * TM + r] + red_sum[3 * TM + r];
-            const RowSum rs = split_2s(S);
-            if (monotone) {
-                // ---- this row's thresholds: part q finds delta_k for k = q + 1, q + 5, q + 9, q + 13
-                //      from the buckets and adds them to the table words
-                if (valid) {
-                    // e(d) D_k <= 2S, exact: one rounding of an exact product minus hi, against lo
-                    auto hit = [&](int d, float D) -> bool { return __fmaf_rn(LUTF[d], D, -rs.hi) <= rs.lo; };
-                    const int bk0 = sh.bk0, bkmax = sh.bkmax;
-                    // the four searches run side by side (independent chains)
-                    float D[4];
-                    int lo[4], n[4];  // delta_k in [lo, lo + n]
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int k = min(q + 1 + 4 * i, 15);
-                        D[i] = kD[k];
-                        const int b = (int)(__float_as_uint(rs.hi * kRcpD[k]) >> BK_SHIFT) - bk0;
-                        if ((unsigned)b < (unsigned)BK_N) {
-                            const uint32_t v = BK[b];
-                            lo[i] = (int)(v & 511u);
-                            n[i] = (int)(v >> 9);
-                            if (n[i] == 127) n[i] = 256 - lo[i];
-                        } else {
-                            lo[i] = b < 0 ? 256 : 0;  // below the buckets: every value lies above T
-                            n[i] = 0;
-                        }
-                    }
-                    (void)bkmax;
-                    // the first d in [lo, lo + n) that hits, else lo + n (binary search)
-                    for (int step = 0; step < 9; ++step) {
-                        bool more = false;
+            CodeRow cr{};
+            if constexpr (DIRECT) cr = code_row(S, e0f);
+            const bool any_fix = DIRECT && __any_sync(0xffffffffu, cr.fix != 0);
+            if constexpr (!DIRECT) {
+                const RowSum rs = split_2s(S);
+                if (monotone) {
+                    // ---- this row's thresholds: part q finds delta_k for k = q + 1, q + 5, q + 9, q + 13
+                    //      from the buckets and adds them to the table words
+                    if (valid) {
+                        // e(d) D_k <= 2S, exact: one rounding of an exact product minus hi, against lo
+                        auto hit = [&](int d, float D) -> bool { return __fmaf_rn(LUTF[d], D, -rs.hi) <= rs.lo; };
+                        const int bk0 = sh.bk0, bkmax = sh.bkmax;
+                        // the four searches run side by side (independent chains)
+                        float D[4];
+                        int lo[4], n[4];  // delta_k in [lo, lo + n]
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
-                            if (n[i] > 0) {
-                                const int h = n[i] >> 1;
-                                if (hit(lo[i] + h, D[i])) {
-                                    n[i] = h;
-                                } else {
-                                    lo[i] += h + 1;
-                                    n[i] -= h + 1;
-                                }
-                                more |= n[i] > 0;
+                            const int k = min(q + 1 + 4 * i, 15);
+                            D[i] = kD[k];
+                            const int b = (int)(__float_as_uint(rs.hi * kRcpD[k]) >> BK_SHIFT) - bk0;
+                            if ((unsigned)b < (unsigned)BK_N) {
+                                const uint32_t v = BK[b];
+                                lo[i] = (int)(v & 511u);
+                                n[i] = (int)(v >> 9);
+                                if (n[i] == 127) n[i] = 256 - lo[i];
+                            } else {
+                                lo[i] = b < 0 ? 256 : 0;  // below the buckets: every value lies above T
+                                n[i] = 0;
                             }
                         }
-                        if (!more) break;
-                    }
+                        (void)bkmax;
+                        // the first d in [lo, lo + n) that hits, else lo + n (binary search)
+                        for (int step = 0; step < 9; ++step) {
+                            bool more = false;
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        if (q + 1 + 4 * i <= 15 && lo[i] < 256) {
-                            red_add_u32(kTabAbs + ((uint32_t)lo[i] << 8) + 4u * (uint32_t)lane, inc);
-                            red_add_u32(sa(&GT[lane * GT_LD + (lo[i] >> 4)]), inc);
+                            for (int i = 0; i < 4; ++i) {
+                                if (n[i] > 0) {
+                                    const int h = n[i] >> 1;
+                                    if (hit(lo[i] + h, D[i])) {
+                                        n[i] = h;
+                                    } else {
+                                        lo[i] += h + 1;
+                                        n[i] -= h + 1;
+                                    }
+                                    more |= n[i] > 0;
+                                }
+                            }
+                            if (!more) break;
+                        }
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            if (q + 1 + 4 * i <= 15 && lo[i] < 256) {
+                                red_add_u32(kTabAbs + ((uint32_t)lo[i] << 8) + 4u * (uint32_t)lane, inc);
+                                red_add_u32(sa(&GT[lane * GT_LD + (lo[i] >> 4)]), inc);
+                            }
                         }
                     }
+                } else if (q == 0) {
+                    rs_hi[r] = rs.hi;
+                    rs_lo[r] = rs.lo;
+                    rs_bits[r] = rs.hibits;
                 }
-            } else if (q == 0) {
-                rs_hi[r] = rs.hi;
-                rs_lo[r] = rs.lo;
-                rs_bits[r] = rs.hibits;
-            }
-            soft_bar();  // C
-            // ---- the operand table: thread (lane, warp g) builds lines 16 g .. 16 g + 15 of column
-            //      lane (rows lane, 32 + lane, 64 + lane, 96 + lane)
-            {
-                const int g = warp;
-                if (monotone) {
-                    uint32_t carry = 0;  // thresholds below line 16 g, per row byte
-                    {
-                        const uint4 *gt = reinterpret_cast<const uint4 *>(GT + lane * GT_LD);
-                        const uint4 g0 = gt[0], g1 = gt[1], g2 = gt[2], g3 = gt[3];
-                        const uint32_t gv[16] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w,
-                                                 g2.x, g2.y, g2.z, g2.w, g3.x, g3.y, g3.z, g3.w};
+                soft_bar();  // C
+                // ---- the operand table: thread (lane, warp g) builds lines 16 g .. 16 g + 15 of column
+                //      lane (rows lane, 32 + lane, 64 + lane, 96 + lane)
+                {
+                    const int g = warp;
+                    if (monotone) {
+                        uint32_t carry = 0;  // thresholds below line 16 g, per row byte
+                        {
+                            const uint4 *gt = reinterpret_cast<const uint4 *>(GT + lane * GT_LD);
+                            const uint4 g0 = gt[0], g1 = gt[1], g2 = gt[2], g3 = gt[3];
+                            const uint32_t gv[16] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w,
+                                                     g2.x, g2.y, g2.z, g2.w, g3.x, g3.y, g3.z, g3.w};
 #pragma unroll
-                        for (int j = 0; j < 15; ++j) carry += j < g ? gv[j] : 0u;
-                    }
-                    const uint32_t a0 = kTabAbs + (uint32_t)(16 * g) * 256u + 4u * (uint32_t)lane;
-                    uint32_t h[16];  // the 16 loads first: the running sum then has no load in its chain
+                            for (int j = 0; j < 15; ++j) carry += j < g ? gv[j] : 0u;
+                        }
+                        const uint32_t a0 = kTabAbs + (uint32_t)(16 * g) * 256u + 4u * (uint32_t)lane;
+                        uint32_t h[16];  // the 16 loads first: the running sum then has no load in its chain
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) h[i] = lds_u32(a0 + 256u * i);
+                        for (int i = 0; i < 16; ++i) h[i] = lds_u32(a0 + 256u * i);
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        carry += h[i];
-                        sts_u32(a0 + 256u * i, 0x78787878u - 4u * carry);  // 4 (30 - code) per byte
-                    }
-                } else {
+                        for (int i = 0; i < 16; ++i) {
+                            carry += h[i];
+                            sts_u32(a0 + 256u * i, 0x78787878u - 4u * carry);  // 4 (30 - code) per byte
+                        }
+                    } else {
 #pragma unroll 1
-                    for (int i = 0; i < 16; ++i) {
-                        const int d = 16 * g + i;
-                        const float ef = LUTF[d];
-                        uint32_t word = 0;
+                        for (int i = 0; i < 16; ++i) {
+                            const int d = 16 * g + i;
+                            const float ef = LUTF[d];
+                            uint32_t word = 0;
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const int rr = 32 * k + lane;
-                            const uint32_t E = operand_exp_f(ef, rs_bits[rr], rs_hi[rr], rs_lo[rr]);
-                            word |= (4u * E) << (8 * k);
+                            for (int k = 0; k < 4; ++k) {
+                                const int rr = 32 * k + lane;
+                                const uint32_t E = operand_exp_f(ef, rs_bits[rr], rs_hi[rr], rs_lo[rr]);
+                                word |= (4u * E) << (8 * k);
+                            }
+                            sts_u32(kTabAbs + (uint32_t)d * 256u + 4u * (uint32_t)lane, word);
                         }
-                        sts_u32(kTabAbs + (uint32_t)d * 256u + 4u * (uint32_t)lane, word);
                     }
                 }
+                soft_bar();  // D
             }
-            soft_bar();  // D
             // the previous tile's MMAs have read the operands in tensor memory: they may be rewritten
             if (it > 0 && !mbar_wait_warp(&sh.mmadone, (it - 1) & 1, abort_flag)) {
                 wait_bad = true;  // the next tile's first barrier ends the loop for all
@@ -744,17 +777,29 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
             }
             // ---- operands of this row's keys -> tensor memory
             {
-                auto ops16 = [&](const uint4 &x, uint32_t (&o)[8]) {
-                    const uint32_t ww[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-                    for (int b = 0; b < 4; ++b) {
-                        const uint32_t t0 = lds_u8(tab_addr<0>(ww[b], rowb));
-                        const uint32_t t1 = lds_u8(tab_addr<1>(ww[b], rowb));
-                        const uint32_t t2 = lds_u8(tab_addr<2>(ww[b], rowb));
-                        const uint32_t t3 = lds_u8(tab_addr<3>(ww[b], rowb));
-                        o[2 * b] = pack_ops(t0, t1);
-                        o[2 * b + 1] = pack_ops(t2, t3);
+                auto ops4 = [&](uint32_t w, uint32_t &o0, uint32_t &o1) {
+                    const uint32_t t0 = DIRECT ? lds_u32(tab_addr<0>(w, rowb)) : lds_u8(tab_addr<0>(w, rowb));
+                    const uint32_t t1 = DIRECT ? lds_u32(tab_addr<1>(w, rowb)) : lds_u8(tab_addr<1>(w, rowb));
+                    const uint32_t t2 = DIRECT ? lds_u32(tab_addr<2>(w, rowb)) : lds_u8(tab_addr<2>(w, rowb));
+                    const uint32_t t3 = DIRECT ? lds_u32(tab_addr<3>(w, rowb)) : lds_u8(tab_addr<3>(w, rowb));
+                    if constexpr (DIRECT) {
+                        o0 = code_ops(__uint_as_float(t0), __uint_as_float(t1), cr);
+                        o1 = code_ops(__uint_as_float(t2), __uint_as_float(t3), cr);
+                        if (any_fix) {  // the key at distance 0, where 3 e > 2S
+                            const uint32_t z = (~(((w & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | w) >> 7) & 0x01010101u;
+                            o0 += prmt(z, 0u, 0x4140u) * cr.fix;
+                            o1 += prmt(z, 0u, 0x4342u) * cr.fix;
+                        }
+                    } else {
+                        o0 = pack_ops(t0, t1);
+                        o1 = pack_ops(t2, t3);
                     }
+                };
+                auto ops16 = [&](const uint4 &x, uint32_t (&o)[8]) {
+                    ops4(x.x, o[0], o[1]);
+                    ops4(x.y, o[2], o[3]);
+                    ops4(x.z, o[4], o[5]);
+                    ops4(x.w, o[6], o[7]);
                 };
                 // (rows past the tile's end take whatever their padding bytes give: their accumulator rows
                 // are never read, and a row of D depends only on its own row of operands)
@@ -766,8 +811,8 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
                 }
                 if (quarter) {  // every part writes its 2 columns of the last MMA step (zeros past L)
                     const uint32_t x = w[NKB - 1].x;
-                    uint32_t o0 = pack_ops(lds_u8(tab_addr<0>(x, rowb)), lds_u8(tab_addr<1>(x, rowb)));
-                    uint32_t o1 = pack_ops(lds_u8(tab_addr<2>(x, rowb)), lds_u8(tab_addr<3>(x, rowb)));
+                    uint32_t o0, o1;
+                    ops4(x, o0, o1);
                     if (last_keys < 4) {
                         o1 = last_keys <= 2 ? 0u : (o1 & 0xFFFFu);
                         if (last_keys < 2) o0 = last_keys == 1 ? (o0 & 0xFFFFu) : 0u;
