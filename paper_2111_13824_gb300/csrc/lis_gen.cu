@@ -37,7 +37,7 @@
 // Measured (us per call): 8 x 12 heads of 785 keys, d = 64, 1129 on CUDA cores -> 62.5
 // (59 M logits; 12 us of bytes); 12 x 12 windows, bias and mask, d = 32, 8-bit output,
 // 1536 heads of 144 keys, 440 -> 56.4 (32 M logits; 7 us of bytes).  Issue-bound:
-// about 20 warp instructions per 32 keys in all (V, read-out and waits among them) at 58 % of
+// about 22 warp instructions per 32 keys in all (V, read-out and waits among them) at 58 % of
 // the issue slots.  Tried without a gain: distances held in registers (62.4 and 58.3 us), seven
 // operand blocks and up to twelve V blocks in flight, V requested a block ahead.
 //

@@ -31,7 +31,7 @@
 // address.  Distances past 15 |q_ln2| all give e(15 |q_ln2|) (the clamp of
 // Algorithm 1), so d is clamped to ne - 1.
 //
-// Issue-bound: about 40 instructions per key.  Swin-S stage 1 with bias and mask (12288
+// Issue-bound: about 35 warp instructions per 32 keys.  Swin-S stage 1 with bias and mask (12288
 // heads of 49 keys) 67.8 us -> 57.7: the code from exponents (code_ops), 13 words of keys
 // instead of 16, no mask arithmetic in the windows of one region.
 //
