@@ -166,7 +166,15 @@ __constant__ float kRcpD[16] = {0.0f,          1.0f / 3.0f,     1.0f / 5.0f,    
 // tensor memory: D at 0 (PACK: the second head's D at 64), the operands P from ta_col on (8 columns
 // per 16 keys), then the row sums of P (zp_V != 0), 16 columns
 __host__ __device__ constexpr int ta_col(bool pack) { return pack ? 2 * TD : TD; }
-__host__ __device__ constexpr int tr_col(int nkb, bool pack) { return ta_col(pack) + 32 * nkb; }
+// Operand regions: two for packed tiles without a table where tensor memory holds them (up to 320 keys), so that a
+// group of 32 rows may write a tile's operands while the MMAs of the tile before wait for the slowest group.
+// us per call, one / two regions, 384 heads: 197 keys 20.5 / 20.0, 257 keys 29.3 / 28.4, 320 keys with 8-bit output
+// 39.7 / 37.8; shorter rows gain nothing (129 keys 15.7 / 15.8).
+__host__ __device__ constexpr int op_bufs(int nkb, bool pack)
+{
+    return pack && nkb <= kDirectBlocks && ta_col(pack) + 64 * nkb + 16 <= 512 ? 2 : 1;
+}
+__host__ __device__ constexpr int tr_col(int nkb, bool pack) { return ta_col(pack) + op_bufs(nkb, pack) * 32 * nkb; }
 __host__ __device__ constexpr int tmem_cols(int nkb, bool pack)
 {
     return tr_col(nkb, pack) + 16 <= 128 ? 128 : tr_col(nkb, pack) + 16 <= 256 ? 256 : 512;
@@ -236,7 +244,8 @@ __device__ __forceinline__ TileInfo next_tile(TileInfo ti, int L, int64_t total)
 }
 
 struct TcShared {
-    uint64_t lload, lfree, afull, mmadone, fin;
+    uint64_t lload, lfree, fin;
+    uint64_t afull[2], mmadone[2];  // of the operand regions
     TcLayout ly;
     IexpC c;
     uint32_t tmem;
@@ -440,8 +449,10 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
     if (tid == 0) {
         mbar_init(&sh.lload, 1);
         mbar_init(&sh.lfree, TSOFT);
-        mbar_init(&sh.afull, TSOFT);
-        mbar_init(&sh.mmadone, 1);
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&sh.afull[b], TSOFT);
+            mbar_init(&sh.mmadone[b], 1);
+        }
         mbar_init(&sh.fin, 1);
         sh.abort_flag = 0;
         sh.rising = 0;
@@ -512,6 +523,9 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
     const int ncta_tiles = (int)((int64_t)(blockIdx.x + 1) * ntiles / gridDim.x - t_begin);
     constexpr int TA = ta_col(PACK);
     constexpr int TR = tr_col(NKB, PACK);
+    constexpr int NB = op_bufs(NKB, PACK);
+    auto region = [](int t) -> int { return NB == 2 ? t & 1 : 0; };  // of the CTA's tile t
+    auto phase = [](int t) -> uint32_t { return (uint32_t)(NB == 2 ? t >> 1 : t) & 1u; };  // of its barriers
 
     if (tid < TSOFT) {
         const int k4 = warp & 3, q = warp >> 2;
@@ -770,13 +784,14 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
                 }
                 soft_bar();  // D
             }
-            // the previous tile's MMAs have read the operands in tensor memory: they may be rewritten
-            if (it > 0 && !mbar_wait_warp(&sh.mmadone, (it - 1) & 1, abort_flag)) {
+            // the MMAs of the tile that last used this operand region have read it: it may be rewritten
+            if (it >= NB && !mbar_wait_warp(&sh.mmadone[region(it - NB)], phase(it - NB), abort_flag)) {
                 wait_bad = true;  // the next tile's first barrier ends the loop for all
                 continue;
             }
             // ---- operands of this row's keys -> tensor memory
             {
+                const uint32_t top = tlane + TA + (uint32_t)region(it) * (32 * NKB);
                 auto ops4 = [&](uint32_t w, uint32_t &o0, uint32_t &o1) {
                     const uint32_t t0 = DIRECT ? lds_u32(tab_addr<0>(w, rowb)) : lds_u8(tab_addr<0>(w, rowb));
                     const uint32_t t1 = DIRECT ? lds_u32(tab_addr<1>(w, rowb)) : lds_u8(tab_addr<1>(w, rowb));
@@ -807,7 +822,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
                 for (int kb = 0; kb < NKB - 1; ++kb) {
                     uint32_t o[8];
                     ops16(w[kb], o);
-                    tmem_st8(tlane + TA + 32 * kb + 8 * q, o);
+                    tmem_st8(top + 32 * kb + 8 * q, o);
                 }
                 if (quarter) {  // every part writes its 2 columns of the last MMA step (zeros past L)
                     const uint32_t x = w[NKB - 1].x;
@@ -817,7 +832,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
                         o1 = last_keys <= 2 ? 0u : (o1 & 0xFFFFu);
                         if (last_keys < 2) o0 = last_keys == 1 ? (o0 & 0xFFFFu) : 0u;
                     }
-                    tmem_st2(tlane + TA + 32 * (NKB - 1) + 2 * q, o0, o1);
+                    tmem_st2(top + 32 * (NKB - 1) + 2 * q, o0, o1);
                 } else if (last_keys > 0) {  // warp-uniform
                     uint32_t o[8];
                     ops16(w[NKB - 1], o);
@@ -828,13 +843,13 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
                         else if (2 * c + 1 == last_keys)
                             o[c] &= 0xFFFFu;
                     }
-                    tmem_st8(tlane + TA + 32 * (NKB - 1) + 8 * q, o);
+                    tmem_st8(top + 32 * (NKB - 1) + 8 * q, o);
                 }
             }
             __syncwarp();
             tmem_wait_st();
             tc_fence_before();
-            mbar_arrive(&sh.afull);
+            mbar_arrive(&sh.afull[region(it)]);
         }
     } else {
         // ---------------- read-out warps (lane quarter eq), with V, the MMA issue and the logits copies
@@ -895,7 +910,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
             }
             bool ok = true;
             if (it > 0) {  // the previous tile's accumulators; then D and the B buffers are free
-                ok = mbar_wait_warp(&sh.mmadone, (it - 1) & 1, abort_flag);
+                ok = mbar_wait_warp(&sh.mmadone[region(it - 1)], phase(it - 1), abort_flag);
                 if (ok) {
                     tc_fence_after();
                     read_out(tp);
@@ -914,9 +929,10 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
             epi_bar();  // D read, B written: this tile's MMAs may run
             if (*ew_stop) break;
             if (warp == TMMA_WARP && elect_one()) {
-                if (mbar_wait(&sh.afull, it & 1, abort_flag)) {
+                if (mbar_wait(&sh.afull[region(it)], phase(it), abort_flag)) {
                     tc_fence_after();
                     const uint64_t ones = smem_desc_plain(sa(ONES), 128, 256);
+                    const uint32_t aop = tmem + TA + (uint32_t)region(it) * (32 * NKB);
                     const int nh = (PACK && ti.nsplit < ti.rows) ? 2 : 1;
                     for (int hh = 0; hh < nh; ++hh) {
                         const int bb = blk0(ti.h0 + hh);
@@ -925,7 +941,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
                         // (address / 16) grows by kBlk / 16 per block
                         uint64_t da = smem_desc(sa(dsm) + blk_off(bm, bb), 1024, 1024);
                         const uint64_t dc = smem_desc(sa(dsm) + bm.bC, 1024, 1024);
-                        uint32_t at = tmem + TA;
+                        uint32_t at = aop;
                         for (int s = 0; s < nsteps; ++s) {
                             mma_f16_ta(dcol, at, da, s != 0);
                             at += 8;
@@ -934,15 +950,15 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
                     }
                     if (p.zp != 0)
                         for (int s = 0; s < nsteps; ++s)
-                            mma_f16_ta(tmem + TR, tmem + TA + 8 * s, ones, s != 0, kIdescOnes);
-                    mma_commit(&sh.mmadone);
+                            mma_f16_ta(tmem + TR, aop + 8 * s, ones, s != 0, kIdescOnes);
+                    mma_commit(&sh.mmadone[region(it)]);
                 } else {
                     *ew_stop = 1;
                 }
             }
         }
         if (it == ncta_tiles && ncta_tiles > 0 && !*ew_stop) {  // the last tile's accumulators
-            if (mbar_wait_warp(&sh.mmadone, (ncta_tiles - 1) & 1, abort_flag)) {
+            if (mbar_wait_warp(&sh.mmadone[region(ncta_tiles - 1)], phase(ncta_tiles - 1), abort_flag)) {
                 tc_fence_after();
                 read_out(ti);
             }
