@@ -466,6 +466,17 @@ __global__ void __launch_bounds__(LTHREADS, 1)
                 if (rank == 0)  // the same; the first CTA's barriers count the bytes of both
                     for (uint32_t j = issued > PF ? issued - PF : 0; j < issued; ++j)
                         mbar_wait(&sh.wfull[j % PF], (j / PF) & 1, abort_flag, false);
+                // The first CTA's commits arrive on the barriers of both.  The cluster barrier at the end orders
+                // threads, not these arrivals: each CTA sees its own last ones here, so that none can land in
+                // shared memory that already belongs to the next CTA of this SM.  (The epilogue waits for every
+                // cfull.  Not while the loop runs: a wait has two seconds.)
+                if (CG == 2) {
+                    for (uint32_t j = issued > PF ? issued - PF : 0; j < issued && ok; ++j)
+                        ok = mbar_wait(&sh.wempty[j % PF], (j / PF) & 1, abort_flag);
+                    for (uint32_t j = issued > LAS ? issued - LAS : 0; j < issued && ok; ++j)
+                        ok = mbar_wait(&sh.aempty[j % LAS], (j / LAS) & 1, abort_flag);
+                    mbar_wait(&sh.fin, 0, abort_flag, false);
+                }
             }
             __syncwarp();
         } else if (warp == LMMA_WARP && rank == 0) {
@@ -688,7 +699,7 @@ __global__ void __launch_bounds__(LTHREADS, 1)
     if (warp < LEPI_WARPS && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");  // stores completed
     tc_fence_before();
     __syncthreads();
-    if (CG == 2) cluster_sync();  // the pair's MMAs and barrier arrivals are over in both CTAs
+    if (CG == 2) cluster_sync();  // both CTAs have seen the pair's last MMAs and arrivals
     tc_fence_after();
     if (warp == 0) {
         if (CG == 1)
