@@ -647,7 +647,8 @@ __global__ void __launch_bounds__(GTHREADS, 1) lis_attn_gen_kernel(const __grid_
             int issued = 0;
             for (int it = 0; it < n; ++it, ti = gen_next(p, ti)) {
                 const int lb = p.nlg == 2 ? it & 1 : 0, use = p.nlg == 2 ? it >> 1 : it;
-                const uint32_t bytes = (uint32_t)(ti.rows * p.ld);
+                // (to the end of the last row's keys: the bytes behind them may not be the caller's to read)
+                const uint32_t bytes = (uint32_t)((ti.rows - 1) * p.ld) + 16u * nsteps;
                 if (it >= p.nlg) {
                     prefetch_l2(p.logits + (size_t)ti.g0 * p.ld, bytes);
                     if (!mbar_wait(&sh.lfree[lb], (uint32_t)(use - 1) & 1u, abort_flag)) break;

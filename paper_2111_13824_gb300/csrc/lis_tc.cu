@@ -865,10 +865,15 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
         auto last_head = [](const TileInfo &t) { return t.nsplit < t.rows ? t.h0 + 1 : t.h0; };
         TileInfo ti = tile_info<PACK>(t_begin, L, p.BH, tpb);
         TileInfo tp = ti;  // the previous tile
+        // bytes of a tile's logits, to the end of its last row's keys: those behind them, up to the stride, may
+        // not be the caller's to read
+        auto tile_bytes = [&](const TileInfo &t) -> uint32_t {
+            return (uint32_t)((t.rows - 1) * p.ld) + 16u * (uint32_t)nsteps;
+        };
         if (warp == TCOPY_WARP && elect_one() && ncta_tiles > 0) {
             prefetch_l2(p.v + (size_t)ti.h0 * L * TD, (uint32_t)(L * TD));
             if (last_head(ti) != ti.h0) prefetch_l2(p.v + (size_t)last_head(ti) * L * TD, (uint32_t)(L * TD));
-            const uint32_t bl = (uint32_t)(ti.rows * p.ld);
+            const uint32_t bl = tile_bytes(ti);
             mbar_expect_tx(&sh.lload, bl);
             bulk_g2s(LG, p.logits + (size_t)ti.g0 * p.ld, bl, &sh.lload);
             ++ncopies;
@@ -896,7 +901,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
                 // the next tile's logits as soon as every softmax thread holds this tile's
                 const TileInfo tn = next_tile<PACK>(ti, L, total);
                 if (mbar_wait(&sh.lfree, it & 1, abort_flag)) {
-                    const uint32_t bl = (uint32_t)(tn.rows * p.ld);
+                    const uint32_t bl = tile_bytes(tn);
                     mbar_expect_tx(&sh.lload, bl);
                     bulk_g2s(LG, p.logits + (size_t)tn.g0 * p.ld, bl, &sh.lload);
                     ++ncopies;
@@ -904,7 +909,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
                         prefetch_l2(p.v + (size_t)last_head(tn) * L * TD, (uint32_t)(L * TD));
                     if (it + 2 < ncta_tiles) {
                         const TileInfo tm = next_tile<PACK>(tn, L, total);
-                        prefetch_l2(p.logits + (size_t)tm.g0 * p.ld, (uint32_t)(tm.rows * p.ld));
+                        prefetch_l2(p.logits + (size_t)tm.g0 * p.ld, tile_bytes(tm));
                     }
                 }
             }

@@ -383,14 +383,17 @@ __global__ void __launch_bounds__(QALL, 1)
             auto idesc = [](int n) -> uint32_t {
                 return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(QM >> 4) << 24);
             };
+            // each copy ends with its last row's codes (16-byte units): the bytes behind them, up to the stride, may
+            // not be the caller's to read
+            const uint32_t d16 = (uint32_t)((d + 15) & ~15);
             auto copy_q = [&](int64_t tt) {
                 const int bq = (int)(tt / tpb), rq = (int)(tt - (int64_t)bq * tpb) * QM;
-                const uint32_t bytes = (uint32_t)(min(QM, L - rq) * p.ld_q);
+                const uint32_t bytes = (uint32_t)((min(QM, L - rq) - 1) * p.ld_q) + d16;
                 mbar_expect_tx(&sh.qload, bytes);
                 bulk_g2s(QST, p.q + ((size_t)bq * L + rq) * p.ld_q, bytes, &sh.qload);
             };
             auto copy_k = [&](int bk) {
-                const uint32_t bytes = (uint32_t)(L * p.ld_k);
+                const uint32_t bytes = (uint32_t)((L - 1) * p.ld_k) + d16;
                 mbar_expect_tx(&sh.kload, bytes);
                 bulk_g2s(KST, p.k + (size_t)bk * L * p.ld_k, bytes, &sh.kload);
             };
