@@ -143,12 +143,16 @@ struct SeqSum {
     }
 
     // adds d[g]^2 of the lanes of groups 0 .. 3, in that order, where the sum stays in its binade (the usual
-    // case: four groups' roundings side by side, one reduction); else does nothing and returns false
+    // case: four groups' roundings side by side, one reduction); else (an infinity or a NaN among them too) does
+    // nothing and returns false
     __device__ __forceinline__ bool add128(const float (&d)[4])
     {
         constexpr unsigned long long kTop = 1ull << 53;
         const uint32_t full = 0xffffffffu;
         const uint32_t below = (1u << (threadIdx.x & 31)) - 1u;
+        // terms of k <= u + 10 can be rounded in 64 bits: the bits of |d| below those of the first exponent past it
+        const int last = min(((u + 10) >> 1) + 150, 254);
+        const uint32_t top = last >= 1 ? (uint32_t)(last + 1) << 23 : 1u;
         unsigned long long n[4];
         bool tie[4], fits = M != 0;
 #pragma unroll
@@ -157,7 +161,7 @@ struct SeqSum {
             int k;
             square(d[g], m, k);
             const int r = min(u - k, 50);  // 50: the term rounds to 0
-            fits = fits && (r >= -10 || m == 0);
+            fits = fits && (__float_as_uint(d[g]) & 0x7FFFFFFFu) < top;
             const unsigned long long t = m + ((1ull << (r & 63)) >> 1);  // (r > 0)
             n[g] = r > 0 ? t >> (r & 63) : m << (-r & 63);  // rounded to nearest, a tie up; or exact
             tie[g] = r > 0 && (n[g] << (r & 63)) == t;
@@ -188,7 +192,9 @@ struct SeqSum {
         return true;
     }
 
-    // adds d^2 of lanes 0 .. 31, in that order, each addition rounded to nearest even (d = 0: no term)
+    // adds d^2 of lanes 0 .. 31, in that order, each addition rounded to nearest even (d = 0: no term).  An
+    // infinite or NaN term takes the fp64 addition, as a crossing; the sum is then an M 2^u as well, whose u (972
+    // or more) no finite term reaches.
     __device__ __forceinline__ void add32(float d)
     {
         constexpr unsigned long long kTop = 1ull << 53;
@@ -208,7 +214,7 @@ struct SeqSum {
                 left &= ~((2u << j) - 1u);
             }
             // the term in units of 2^u: n, its floor where it is a tie (capped: a sum of 2^53 is a crossing)
-            const int sh = k - u;
+            const int sh = isfinite(d) ? k - u : 11;
             unsigned long long n = 0;
             bool tie = false;
             if ((left >> lane) & 1u) {
