@@ -9,7 +9,8 @@
 //   2. every block folds the partials into s, zp (Eqs. 8-9), then a warp per
 //      (channel, factor) sums the squared quantization error of Eq. 10 over
 //      the rows, in ascending row order, in fp64, and the block's channels
-//      take the smallest factor with the least error.
+//      take the smallest factor with the least error.  Few rows (the rule is at launch_sse): a
+//      thread per sum.
 //
 // The fp64 sums.  The order fixes the rounding of every step, and fp64 is slow
 // on this GPU (one thread per sum took 1.0 ms for 6304 rows of 384 channels,
@@ -266,6 +267,80 @@ struct SeqSum {
 constexpr int kSseRows = 1024, CH = 2;
 constexpr int kSseFactors = 4;   // factors per block
 
+// The range (min, max) of the partials part[nparts], to every thread of the block
+__device__ __forceinline__ void fold_range(const float *__restrict__ part, int nparts, float &mn, float &mx)
+{
+    __shared__ float2 red[32];
+    const int tid = threadIdx.x, nthreads = blockDim.x;
+    mn = FLT_MAX, mx = -FLT_MAX;
+    for (int i = tid; i < nparts; i += nthreads) {
+        mn = fminf(mn, part[2 * i]);  // (a caller's range need not be 8-byte aligned)
+        mx = fmaxf(mx, part[2 * i + 1]);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    }
+    if ((tid & 31) == 0) red[tid >> 5] = make_float2(mn, mx);
+    __syncthreads();
+    for (int w = 0; w < nthreads / 32; ++w) {
+        mn = fminf(mn, red[w].x);
+        mx = fmaxf(mx, red[w].y);
+    }
+}
+
+// The smallest factor with the least of a channel's errors err[0], err[step] .. err[K step]
+__device__ __forceinline__ uint8_t least(const double *err, int step, int K)
+{
+    int ba = 0;
+    for (int k = 1; k <= K; ++k)
+        if (err[k * step] < err[ba * step]) ba = k;
+    return (uint8_t)ba;
+}
+
+// Eq. 10 for few rows: a thread per (channel, factor), 32 channels a block, a warp per factor.  Bound by the chain
+// of fp64 additions, 0.16 us a row, up to about 20 thousand sums; above by the fp64 pipe.
+__global__ void __launch_bounds__(32 * kSseFactors)
+    calib_sse_few_kernel(const float *__restrict__ x, int64_t rows, int C, int64_t ld, int K,
+                         const float *__restrict__ part, int nparts, float *__restrict__ s_out,
+                         int32_t *__restrict__ zp_out, double *__restrict__ sse, uint8_t *__restrict__ alpha)
+{
+    __shared__ double err[kSseFactors][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float mn, mx, s0, s;
+    int32_t zp;
+    fold_range(part, nparts, mn, mx);
+    calib_scale(mn, mx, K, s0, s, zp);
+    if (s_out && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
+        *s_out = s;
+        *zp_out = zp;
+    }
+    const int c = blockIdx.x * 32 + lane, a = blockIdx.y * kSseFactors + warp;
+    if (c < C && a <= K) {
+        const float up = pow2f(K - a);                 // 1 / (2^(a-K))
+        const float sa = __fmul_rn(s0, pow2f(a - K));  // 2^a s, exact
+        const float lo = (float)(-zp), hi = (float)(255 - zp);
+        double acc = 0.0;
+        for (int64_t r0 = 0; r0 < rows; r0 += 4) {  // four rows' loads and errors side by side
+            float v[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[i] = __ldg(x + min(r0 + i, rows - 1) * ld + c);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float q = fminf(fmaxf(rintf(__fmul_rn(__fdiv_rn(v[i], s0), up)), lo), hi);
+                const double d = (double)__fsub_rn(v[i], __fmul_rn(q, sa));
+                if (r0 + i < rows) acc = __dadd_rn(acc, __dmul_rn(d, d));
+            }
+        }
+        sse[(int64_t)c * (K + 1) + a] = acc;
+        err[warp][lane] = acc;
+    }
+    if (alpha) {
+        __syncthreads();
+        if (warp == 0 && c < C) alpha[c] = least(&err[0][lane], 32, K);
+    }
+}
+
 // Eq. 10 for two channels and up to four factors per block, a warp per (channel, factor): sum over rows of
 // (x - clip(rint(x / (2^a s)), -zp, 255-zp) * 2^a s)^2 in fp64, ascending rows.
 // x / (2^a s) is computed as (x / s0) * 2^(K-a): scaling a correctly rounded
@@ -280,24 +355,10 @@ __global__ void __launch_bounds__(32 * CH * kSseFactors)
 {
     // x and x / s0 (one division for the factors)
     __shared__ float tile[2][CH][kSseRows + 4], tdiv[2][CH][kSseRows + 4];
-    __shared__ float2 red[32];
     __shared__ double err[CH][kSseFactors];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nthreads = blockDim.x;
-    float mn = FLT_MAX, mx = -FLT_MAX;
-    for (int i = tid; i < nparts; i += nthreads) {
-        mn = fminf(mn, part[2 * i]);  // (a caller's range need not be 8-byte aligned)
-        mx = fmaxf(mx, part[2 * i + 1]);
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    }
-    if (lane == 0) red[warp] = make_float2(mn, mx);
-    __syncthreads();
-    for (int w = 0; w < nthreads / 32; ++w) {
-        mn = fminf(mn, red[w].x);
-        mx = fmaxf(mx, red[w].y);
-    }
+    float mn, mx;
+    fold_range(part, nparts, mn, mx);
     float s0, s;
     int32_t zp;
     calib_scale(mn, mx, K, s0, s, zp);
@@ -363,12 +424,7 @@ __global__ void __launch_bounds__(32 * CH * kSseFactors)
     }
     if (alpha) {
         __syncthreads();
-        if (tid < CH && c0 + tid < C) {
-            int ba = 0;
-            for (int k = 1; k <= K; ++k)
-                if (err[tid][k] < err[tid][ba]) ba = k;
-            alpha[c0 + tid] = (uint8_t)ba;
-        }
+        if (tid < CH && c0 + tid < C) alpha[c0 + tid] = least(err[tid], 1, K);
     }
 }
 
@@ -377,15 +433,7 @@ __global__ void calib_argmin_kernel(const double *__restrict__ sse, int C, int K
 {
     int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= C) return;
-    const double *e = sse + (int64_t)c * (K + 1);
-    double best = e[0];
-    int ba = 0;
-    for (int a = 1; a <= K; ++a)
-        if (e[a] < best) {
-            best = e[a];
-            ba = a;
-        }
-    alpha[c] = (uint8_t)ba;
+    alpha[c] = least(sse + (int64_t)c * (K + 1), 1, K);
 }
 
 // Eq. 7.  x / (2^alpha s) = (x / s) * 2^-alpha by the same scaling argument.
@@ -450,12 +498,23 @@ namespace {
 // The error sums (and s, zp, alpha where not null) from the range partials.  A plain launch: with
 // programmatic serialization the blocks start while the range kernel's still hold most SMs and stack up on
 // the others (6304 x 192: 141 us against 62).
+//
+// The rule: a warp's sum costs about 7 us and 2 ns per sum whatever the rows (its start crosses a binade every few
+// rows, and a stage holds 1024), a thread's 0.16 us a row.  us of the sums alone, warps / threads: 8 channels,
+// K = 3: 32 rows 8.5 / 7.4, 48 rows 9.1 / 9.7; 1024, K = 3: 64 rows 15.2 / 12.6, 128 rows 16.2 / 22.8; 4096,
+// K = 3: 32 rows 40.2 / 7.5, 256 rows 61.8 / 44.0, 512 rows 83.7 / 85.6; 8192, K = 7: 512 rows 298 / 224.
 cudaError_t launch_sse(const float *x, int64_t rows, int C, int64_t ld_x, int K, const float *part, int nparts,
                        float *s, int32_t *zp, double *sse, uint8_t *alpha, cudaStream_t st)
 {
     const int nf = K + 1 < kSseFactors ? K + 1 : kSseFactors, ny = (K + kSseFactors) / kSseFactors;
-    const dim3 g((unsigned)((C + CH - 1) / CH), (unsigned)ny), b((unsigned)(32 * CH * nf));
-    calib_sse_kernel<<<g, b, 0, st>>>(x, rows, C, ld_x, K, part, nparts, s, zp, sse, ny > 1 ? nullptr : alpha);
+    uint8_t *al = ny > 1 ? nullptr : alpha;
+    if (rows < 36 + (int64_t)C * (K + 1) / 64) {
+        const dim3 g((unsigned)((C + 31) / 32), (unsigned)ny);
+        calib_sse_few_kernel<<<g, 32 * nf, 0, st>>>(x, rows, C, ld_x, K, part, nparts, s, zp, sse, al);
+    } else {
+        const dim3 g((unsigned)((C + CH - 1) / CH), (unsigned)ny);
+        calib_sse_kernel<<<g, 32 * CH * nf, 0, st>>>(x, rows, C, ld_x, K, part, nparts, s, zp, sse, al);
+    }
     return cudaGetLastError();
 }
 
