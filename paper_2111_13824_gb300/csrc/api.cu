@@ -82,6 +82,18 @@ void forget_smem(SmemReady &ready)
     if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64) ready[dev].store(0, std::memory_order_relaxed);
 }
 
+void *tensor_map_encoder()
+{
+    static void *const encode = [] {  // (initialized by one thread, the others wait)
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        const cudaError_t e =
+            cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q);
+        return e == cudaSuccess && q == cudaDriverEntryPointSuccess ? fn : nullptr;
+    }();
+    return encode;
+}
+
 int record_error(int code, const char *msg)
 {
     if (code == FQVIT_OK) return ok();

@@ -38,6 +38,10 @@ cudaError_t launch_prepared(const void *kernel, size_t dynamic, SmemReady &ready
     }
 }
 
+// The driver's cuTensorMapEncodeTiled (version 12000), NULL when it has none.  Looked up once; threads that
+// come while the first is at it wait for its result.
+void *tensor_map_encoder();
+
 // Programmatic dependent launch.  The step's kernels are launched with programmatic stream
 // serialization: the next kernel's CTAs may start (and run their set-up: barriers, tensor
 // memory, tables computed from arguments) while the previous kernel's last CTAs finish.  Every

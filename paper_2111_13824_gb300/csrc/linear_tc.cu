@@ -749,17 +749,7 @@ __global__ void __launch_bounds__(256) bytes_to_half_kernel(const uint8_t *src, 
 bool tensor_map(CUtensorMap *tm, const void *ptr, bool half, int64_t rows, int cols, int64_t ld, int box_cols,
                 int box_rows, CUtensorMapSwizzle swizzle)
 {
-    static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
-        void *fn = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-    }
+    const auto encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(tensor_map_encoder());
     if (!encode) return false;
     memset(tm, 0, sizeof(*tm));
     const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};

@@ -542,17 +542,7 @@ cudaError_t qk_launch(const QkParams &p, const CUtensorMap &tm, size_t smem, int
 // 128-byte swizzle.  False when the driver's encoder is unavailable or rejects the shape.
 bool logits_tensor_map(CUtensorMap *tm, int8_t *out, int64_t BH, int L, int64_t ld)
 {
-    static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
-        void *fn = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-    }
+    const auto encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(tensor_map_encoder());
     if (!encode) return false;
     const cuuint64_t dims[3] = {(cuuint64_t)ld, (cuuint64_t)L, (cuuint64_t)BH};
     const cuuint64_t strides[2] = {(cuuint64_t)ld, (cuuint64_t)ld * (cuuint64_t)L};
