@@ -219,7 +219,7 @@ bool lis_attention_win_eligible(const LisArgs &a, const AttnVArgs &b);
 cudaError_t launch_lis_attention_win(const LisArgs &a, const AttnVArgs &b, cudaStream_t st);
 cudaError_t read_clear_win_status(int *status);
 
-// tensor-core fused path for the rows neither of these takes: up to 1024 keys without a bias, up to
+// tensor-core fused path for the rows neither of these takes: 25 to 1024 keys without a bias, up to
 // 256 with one (and a mask) (lis_gen.cu)
 bool lis_attention_gen_eligible(const LisArgs &a, const AttnVArgs &b);
 cudaError_t launch_lis_attention_gen(const LisArgs &a, const AttnVArgs &b, cudaStream_t st);

@@ -2,7 +2,8 @@
 // the BitShift attention times values (Eq. 15) on CUDA cores: the softmax and
 // the product on their own (codes in memory), the fused form where no
 // tensor-core kernel takes the shape (codes written too, a mask without a bias,
-// windows above 256 keys, unaligned rows), and the choice between them.
+// windows above 256 keys, rows below 25 keys that the short-row kernel does not
+// take, unaligned rows), and the choice between them.
 //
 // i-exp.  For a logit scale s the values e(q~) for every q~ in [-287, 0]
 // (int8 logits, plus an int8 relative-position bias) are tabulated in

@@ -1,9 +1,10 @@
 // lis_gen.cu -- fused Log-Int-Softmax + BitShift attention times values on the
 // tcgen05 tensor cores for the rows that the other two tensor-core kernels do
-// not take: rows of up to 1024 keys with head dimension 32 or 64 (lis_tc.cu
+// not take: rows of 25 to 1024 keys with head dimension 32 or 64 (lis_tc.cu
 // holds at most 592 keys and d = 64), and windows of up to 256 keys with a
 // relative-position bias and a shifted-window mask (lis_win.cu: 64 keys).
-// These ran on CUDA cores before (lis.cu), a multiply-add per key and value.
+// These ran on CUDA cores before (lis.cu), a multiply-add per key and value; shorter
+// rows still do (GMIN_L).
 //
 // The product is the one of lis_tc.cu: acc = P V - zp_V (P 1) with
 // P[i][j] = 2^(15 - code_ij), exact in fp16 with fp32 accumulation.  Nothing of
@@ -63,6 +64,11 @@ constexpr int GTHREADS = 32 * (GCOPY_WARP + 1);
 constexpr int GPS = 4;                  // operand blocks in tensor memory (32 columns each)
 constexpr int GVS = 3;                  // V blocks in shared memory (64 keys x 128 bytes)
 constexpr uint32_t GV_BYTES = 64 * 128;
+// Rows below this many keys stay on CUDA cores: a head is a tile, whose fixed cost (its barriers, the read-out of 128
+// accumulator rows) does not shrink with the row.  us per call, CUDA cores / this kernel, d = 64, 3000 heads: 4 keys 15.0
+// / 40.6, 16 keys 32.8 / 41.0, 24 keys 50.3 / 44.1, 32 keys 75.7 / 43.3; 3072 windows with a bias: 16 keys 45.7 / 53.8, 25
+// keys 77.9 / 56.9; d = 32, 700 heads: 24 keys 11.9 / 12.7, 26 keys 14.0 / 12.8.
+constexpr int GMIN_L = 25;
 constexpr uint32_t kSmemOptin = 232448;
 // tensor memory: accumulators [tile parity][head of the tile] of 64 columns, operands, row sums [parity]
 constexpr uint32_t G_TA = 256, G_TR = G_TA + 32 * GPS, G_TMEM = 512;
@@ -719,7 +725,8 @@ cudaError_t gen_launch_d(const LisArgs &a, const GenParams &p, uint32_t smem, in
 
 bool lis_attention_gen_eligible(const LisArgs &a, const AttnVArgs &b)
 {
-    if (a.codes != nullptr || a.rowsum != nullptr || a.L > 1024 || !(b.d == 32 || b.d == 64)) return false;
+    if (a.codes != nullptr || a.rowsum != nullptr || a.L < GMIN_L || a.L > 1024 || !(b.d == 32 || b.d == 64))
+        return false;
     if (a.bias ? a.L > 256 : a.region != nullptr) return false;
     if (a.ld_logit % 16 != 0 || ((uintptr_t)a.logits % 16) != 0) return false;
     if (b.ld_v % 16 != 0 || ((uintptr_t)b.v % 16) != 0) return false;
