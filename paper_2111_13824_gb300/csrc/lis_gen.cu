@@ -763,7 +763,7 @@ cudaError_t launch_lis_attention_gen(const LisArgs &a, const AttnVArgs &b, cudaS
     p.mask_c = a.mask_value < -1024 ? 1024 : -a.mask_value;
     p.out8 = b.out8;
     p.ld_out8 = b.ld_out8;
-    p.rq = requant8_of(b.rq_n1, b.rq_n2, b.rq_zp, b.zp_v);
+    p.rq = requant8_of(b.rq_n1, b.rq_n2, b.rq_zp, b.zp_v, a.L);
     uint32_t smem;
     if (!gen_layout(a, p, smem)) return cudaErrorInvalidConfiguration;
     const int64_t ntiles = p.pack ? (b.BH * a.L + GM - 1) / GM : b.BH * ((a.L + GM - 1) / GM);

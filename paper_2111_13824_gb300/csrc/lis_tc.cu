@@ -1031,7 +1031,7 @@ cudaError_t launch_lis_attention_tc(const LisArgs &a, const AttnVArgs &b, cudaSt
     const bool pack = use_pack(a.L);
     const uint32_t smem = tc_smem_bytes(a.L, a.ld_logit, pack);
     TcParams p{a.logits, a.ld_logit, b.v, b.acc, b.BH, a.L, b.zp_v, iexp_consts_host(a.s_logit),
-               b.out8, b.ld_out8, requant8_of(b.rq_n1, b.rq_n2, b.rq_zp, b.zp_v), smem};
+               b.out8, b.ld_out8, requant8_of(b.rq_n1, b.rq_n2, b.rq_zp, b.zp_v, a.L), smem};
     const int64_t ntiles = pack ? (b.BH * a.L + TM - 1) / TM : b.BH * ((a.L + TM - 1) / TM);
     const int grid = (int)(ntiles < sm_count() ? ntiles : sm_count());
     const bool se = small_iexp(p.ic);

@@ -582,7 +582,7 @@ cudaError_t launch_lis_attention_win(const LisArgs &a, const AttnVArgs &b, cudaS
 {
     const bool bias = a.bias != nullptr;
     WinParams p{a.logits, a.ld_logit, b.v, b.ld_v, b.acc, b.ld_acc, a.bias, a.heads, a.window, b.BH, a.L, b.zp_v,
-                iexp_consts_host(a.s_logit), 0, 0, b.out8, b.ld_out8, requant8_of(b.rq_n1, b.rq_n2, b.rq_zp, b.zp_v),
+                iexp_consts_host(a.s_logit), 0, 0, b.out8, b.ld_out8, requant8_of(b.rq_n1, b.rq_n2, b.rq_zp, b.zp_v, a.L),
                 a.region, a.n_windows, a.mask_value < -1024 ? 1024 : -a.mask_value};
     const int mwin = a.region ? a.n_windows : 0;
     p.ne = win_table_entries(p.ic, bias);
