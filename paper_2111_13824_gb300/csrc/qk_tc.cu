@@ -206,7 +206,7 @@ __device__ __forceinline__ void convert_rows(const unsigned char *src, int64_t l
 // BULK: Q and K rows reach shared memory as int8 by bulk copies one tile (one head) ahead of
 // their conversion (strides of at most 64 bytes, multiples of 16), and each chunk's 128 x 128
 // output bytes leave through one of QNST staging buffers (128-byte swizzle) by a tensor store
-// of the logits viewed as [BH][L][ld] (rows past L and bytes past ld clipped), so the drain of
+// of the logits viewed as [BH][L][ld] (rows past L and bytes past ld clipped; qk_bulk: the chunks cover ld), so the drain of
 // one chunk overlaps the work on the next.  Else each thread loads its codes from global
 // memory as it converts them, and the tile's output is copied out from a shared-memory tile.
 template <bool FOLD, bool BULK>
@@ -554,11 +554,13 @@ bool logits_tensor_map(CUtensorMap *tm, int8_t *out, int64_t BH, int L, int64_t 
 }
 
 // Bulk copies of the operands (16-byte aligned rows of at most 64 bytes) and tensor stores of the
-// output (rows and row strides of at least one 128 x 128 box)
+// output (rows and row strides of at least one 128 x 128 box; a stride within the boxes of the keys' chunks, for
+// the bytes behind them, up to the stride, are zeros that no box would write)
 bool qk_bulk(const QkArgs &a)
 {
     return a.ld_q % 16 == 0 && a.ld_k % 16 == 0 && a.ld_q <= 64 && a.ld_k <= 64 && ((uintptr_t)a.q % 16) == 0 &&
            ((uintptr_t)a.k % 16) == 0 && a.L >= QM && a.ld_logit >= QNC &&
+           a.ld_logit <= (a.L + QNC - 1) / QNC * QNC &&
            qk_smem_bytes(a.ld_logit, true) + kQkStaticSmem <= 232448;
 }
 
