@@ -249,7 +249,7 @@ struct TcShared {
     TcLayout ly;
     IexpC c;
     uint32_t tmem;
-    int bk0, bkmax;  // bucket number of table entry 0, and of the last entry
+    int bk0;  // bucket number of table entry 0
     int abort_flag;
     int rising;   // some i-exp value exceeds the one before it (floored constants)
     int stop[4];  // set (never cleared) by a softmax thread whose wait gave up, for the threads that meet it
@@ -488,7 +488,6 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
     }
     if (tid == 0) {
         const int bkmax = (int)(__float_as_uint(LUTF[0] * (1.0f + 0x1p-20f)) >> BK_SHIFT);
-        sh.bkmax = bkmax;
         sh.bk0 = bkmax - (BK_N - 1);
     }
     __syncthreads();  // the copies of the i-exp values read, rising, the bucket range
@@ -691,7 +690,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
                     if (valid) {
                         // e(d) D_k <= 2S, exact: one rounding of an exact product minus hi, against lo
                         auto hit = [&](int d, float D) -> bool { return __fmaf_rn(LUTF[d], D, -rs.hi) <= rs.lo; };
-                        const int bk0 = sh.bk0, bkmax = sh.bkmax;
+                        const int bk0 = sh.bk0;
                         // the four searches run side by side (independent chains)
                         float D[4];
                         int lo[4], n[4];  // delta_k in [lo, lo + n]
@@ -710,7 +709,6 @@ __global__ void __launch_bounds__(TTHREADS, 1) lis_attn_tc_kernel(TcParams p)
                                 n[i] = 0;
                             }
                         }
-                        (void)bkmax;
                         // the first d in [lo, lo + n) that hits, else lo + n (binary search)
                         for (int step = 0; step < 9; ++step) {
                             bool more = false;
@@ -1005,11 +1003,14 @@ template <int NKB>
 cudaError_t tc_launch_e(bool small_e, bool pack, const TcParams &p, size_t smem, int grid, cudaStream_t st)
 {
     if constexpr (NKB <= kPackMaxBlocks && NKB >= 2) {
-        if (pack)
+        if (pack || NKB > 2)  // (use_pack holds for every row of 3 to kPackMaxBlocks blocks)
             return small_e ? tc_launch<NKB, true, true>(p, smem, grid, st)
                            : tc_launch<NKB, false, true>(p, smem, grid, st);
     }
-    return small_e ? tc_launch<NKB, true, false>(p, smem, grid, st) : tc_launch<NKB, false, false>(p, smem, grid, st);
+    if constexpr (NKB <= 2 || NKB > kPackMaxBlocks)
+        return small_e ? tc_launch<NKB, true, false>(p, smem, grid, st)
+                       : tc_launch<NKB, false, false>(p, smem, grid, st);
+    return cudaErrorInvalidConfiguration;
 }
 
 // Whether every i-exp value of the scale is below 2^28: the largest is e(0) = (q_b^2 + q_c) 2^15.

@@ -154,12 +154,6 @@ __device__ __forceinline__ uint32_t operand_exp_f(float ef, int G, float hi, flo
     return (uint32_t)max(31 - k + (int)le, 15);
 }
 
-// the same for an integer i-exp value (exact in fp32: at most 16 significant bits)
-__device__ __forceinline__ uint32_t operand_exp(uint32_t e, int G, float hi, float lo)
-{
-    return operand_exp_f(__uint2float_rn(e), G, hi, lo);
-}
-
 
 // 2S = hi + lo with hi = fp32(2S) rounded to nearest even and lo exact (|lo| < 2^19), from
 // integer operations only (the same values as the fp32 conversions of make_rowsum)
@@ -251,13 +245,6 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t *b, uint32_t parity, vol
     return __all_sync(0xFFFFFFFFu, mbar_wait(b, parity, abort_flag));
 }
 
-__device__ __forceinline__ uint32_t lds32(uint32_t a)
-{
-    uint32_t v;
-    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
-    return v;
-}
-
 // byte permute with the sign-replicate selector bit honoured
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel)
 {
@@ -288,15 +275,6 @@ __device__ __forceinline__ void tmem_st2(uint32_t taddr, uint32_t r0, uint32_t r
 {
     __syncwarp();
     asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1,%2};" ::"r"(taddr), "r"(r0), "r"(r1) : "memory");
-}
-
-// warp-collective (.sync.aligned): the whole warp, converged, writes its 32 lanes (4 columns)
-__device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint32_t (&r)[4])
-{
-    __syncwarp();
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(taddr), "r"(r[0]), "r"(r[1]),
-                 "r"(r[2]), "r"(r[3])
-                 : "memory");
 }
 
 // warp-collective (.sync.aligned): the whole warp, converged, writes its 32 lanes
