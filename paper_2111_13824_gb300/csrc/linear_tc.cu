@@ -40,12 +40,13 @@
 // 32-row staging areas by tensor stores (16-byte stores at the rows' stride
 // cost fc1 of ViT-L/384 20 us of 129).
 //
-// Measured (us per call, back to back; before -> now), M = 18464: QKV (3072 x
-// 1024) 118.2 -> 73.4, projection (1024 x 1024) 46.8 -> 30.9, fc1 (4096 x 1024)
-// 148.0 -> 96.1 (1612 TFLOP/s), fc2 (1024 x 4096) 174.7 -> 94.3 (1642 TFLOP/s);
-// M = 1576: 2304 x 768 17.1 -> 9.5, 768 x 3072 29.1 -> 14.7; M = 197: 192 x 192
-// 8.8 -> 3.6.  What bounds the large ones now is the conversion's latency (a
-// step takes 518 cycles, its MMAs 384; without the conversion 492).
+// Measured (us per call, back to back in a graph; the earlier form -> this one), M =
+// 18464: QKV (3072 x 1024) 118.2 -> 74.7, projection (1024 x 1024) 46.8 -> 31.5, fc1
+// (4096 x 1024) 148.0 -> 98.4 (1574 TFLOP/s), fc2 (1024 x 4096) 174.7 -> 97.7 (1585);
+// M = 1576: 2304 x 768 17.1 -> 9.9, 768 x 3072 29.1 -> 16.2; M = 197: 192 x 192
+// 8.8 -> 4.2.  (Up to 7 % more on some GPUs.)  A step of the large ones takes 518
+// cycles, its MMAs 384.  Timed without the conversion 492, so that accounts for 26 of
+// the difference; what takes the other 108 is not known.
 //
 // Requantization.  Where every channel of the CTA allows it (see channel_entry)
 // y is one fused multiply-add rounded down and a saturating conversion:
@@ -304,7 +305,9 @@ __device__ __forceinline__ void bytes_to_h16(const uint4 &w, __half2 z, uint32_t
     }
 }
 
-// 16 bytes of a row of x from column k on; columns at or past K read as 0 (the weights are 0 there)
+// 16 bytes of a row of x from column k on; columns at or past K read as 0 (the weights are 0 there).
+// Rows that are not multiples of 16 bytes (every contiguous x with K = 8 mod 16) come this way: 18464 x 4096
+// x 1016 124 us (98 at K = 1024; the earlier form with its copy of x 196), 8200 x 1536 x 1000 28.0 (45.2).
 __device__ __forceinline__ uint4 load_x16(const uint8_t *row, int k, int K)
 {
     uint2 a = make_uint2(0, 0), b = make_uint2(0, 0);  // K and the stride are multiples of 8

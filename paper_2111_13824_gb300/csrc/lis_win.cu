@@ -98,8 +98,10 @@ __device__ __forceinline__ uint32_t lut_off(uint32_t dpair, uint32_t lane4)
     return prmt(dpair, lane4, SEL);
 }
 
-// NW: words of four keys of a row, ceil(L / 4) <= NW (13: exactly, the 49 keys of a 7 x 7 window; with whole
-// 16-key chunks a fourth of their pairs were padding).  MASK (with BIAS): the shifted-window mask; windows of
+// NW: words of four keys of a row, ceil(L / 4) <= NW: whole 16-key chunks, and 13, the exact count of 49 .. 52
+// keys, for the 7 x 7 window, where with whole chunks a fourth of the pairs were padding.  (Other lengths with
+// words to spare, 17-28, 33-44 and 53-60 keys, form the pairs of all their chunks; no window but 5 x 5 and
+// 6 x 6 is among them.)  MASK (with BIAS): the shifted-window mask; windows of
 // one region (all but the last row and column of the map) skip its arithmetic.  Logits then sit in the 16-bit lanes as v = q + bias + 1280 - (masked ? m_c : 0) with m_c the
 // mask magnitude clamped to 1024: a key masked by more still lands below every unmasked key (the
 // query's own key is never masked, v >= 1024) at a distance above 510 >= the table's last entry,
